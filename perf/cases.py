@@ -254,7 +254,6 @@ def prepare(case, seed):
     s.cache = sva.Cache(_geometry(c, own, other), device=torch.device(DEV))
     s.cache.set_workspace(torch.empty(s.cache.workspace_bytes(), dtype=torch.uint8, device=DEV))
     slot = {st: s.cache.bind(*st) for st in own + other}
-    s.slots = [slot[st] for st in own]
     within = sva.WITHIN_FRAME_CAUSAL if c["causal"] else sva.WITHIN_BIDIRECTIONAL
     s.nodes = sva.make_nodes([dict(seq=q, chunk=b, level=j, own_slot=slot[(q, b, j)],
                                    ctx=[slot[t] for t in ctx], within=within)
@@ -270,13 +269,9 @@ def prepare(case, seed):
     if c["kind"].startswith(("layer", "attend")):
         s.out = torch.empty_like(s.q)
         s.lse = torch.empty((n, H, T), dtype=torch.float32, device=DEV)
+    pool = s.cache.slot_pool()
+    s.written = [pool[slot[st]][:, :, :T] for st in own]   # K' and V of the nodes' own states, in the cache
     return s
-
-
-def _written(s):
-    """K' and V of the nodes' own states, as the cache holds them."""
-    pool, T = s.cache.slot_pool(), _tokens(s.c)
-    return [pool[k][:, :, :T] for k in s.slots]
 
 
 def run(state):
@@ -284,16 +279,16 @@ def run(state):
     kind = c["kind"]
     if kind == "write":
         s.cache.rope_kv_write(s.nodes, i.k, i.v)
-        return _written(s)
+        return s.written
     if kind == "write_norm":
         s.cache.rope_kv_write_qknorm(s.nodes, i.k, i.v, None, i.gk, None, EPS)
-        return _written(s)
+        return s.written
     if kind == "project":
         s.cache.qkv_project(i.x, i.w, i.b, s.q, s.k, s.v)
         return [s.q, s.k, s.v]
     if kind == "project_rope":
         s.cache.qkv_project_rope(s.nodes, i.x, i.w, i.b, s.q)
-        return [s.q] + _written(s)
+        return [s.q] + s.written
     if kind == "layer":
         s.cache.qkv_project_rope(s.nodes, i.x, i.w, i.b, s.q)
     elif kind == "layer_norm":
