@@ -21,7 +21,7 @@
 //              each; S from TMEM, fp32 online softmax in the log2 domain with
 //              a lazy rescale of O, P written back over S as bf16; then the
 //              epilogue (O / l to bf16 global, optional LSE).
-// TMEM columns: S0 [0,128), S1 [128,256), O0 [256, 256+d), O1 [384, 384+d).
+// TMEM columns (d = 128): S0 [0,128), S1 [128,256), O0 [256,384), O1 [384,512).
 // Each issuer's order per key tile i is PV_b,i then S_b,i+1, so the softmax of
 // either query tile has the other tile's PV and S (two 128x128x128 MMAs) to
 // hide behind.  A tcgen05.mma costs its issuing warp nearly as long as the
@@ -31,6 +31,28 @@
 // the MMAs to issue.  A commit that completes S_b of tile i also implies PV_b
 // of tile i-1 is complete (one issuer per tile, MMAs of a thread execute in
 // issue order), so the rescale of O_b needs no extra barrier.
+//
+// Head dimension 64 halves the MMAs of a key tile (1024 tensor cycles instead
+// of 2048) but not its softmax, so the loop above, whose period is two
+// softmaxes one after the other plus the hand-overs, ran as slowly as at 128
+// (2300 cycles a key tile, tensor pipe 40% busy, MUFU 42%, no unit near its
+// limit).  There:
+//   - warps 4-7 own query tile 0 and warps 8-11 query tile 1, a thread per row
+//     with all 128 keys: two independent softmax chains, in opposite phase
+//     because of the buffer rotation below, so that one's exponentials run
+//     while the other waits for loads and barriers (in phase they contend for
+//     the MUFU and then idle together: 2700 cycles);
+//   - O needs 64 columns a tile, so three S buffers fit: S columns [0,384) by
+//     step n = (key tile, query tile) mod 3, O0 [384,448), O1 [448,512).  The
+//     S of a step are issued one and a half key tiles before their softmax,
+//     right behind the PV that reads the buffer they overwrite;
+//   - both issuers together need all the issue slots they can get: an MMA run
+//     is issued under one election (an election per MMA held a single issuer
+//     at 1450 cycles a step), the even steps' PV by warp 1, the odd ones' by
+//     warp 3, and the V stages are freed by their commits.
+// 2 nodes x 16 heads x 2160 tokens over 10800 keys: 217 -> 176 us (880 -> 1085
+// TFLOP/s).  What bounds it now is the chain of one step: S wait 190 cycles,
+// TMEM load 200, max and vote 230, exponentials 780, P store and hand-over 150.
 // A unit may be split into n_split contiguous key ranges (when there are too
 // few units to fill the GPU's waves): each split CTA writes its normalised
 // partial O with its row max and sum to the workspace and bumps the unit's
@@ -59,18 +81,34 @@ struct AttnCfg {
   static constexpr int kBoxes = D / 64;
   static constexpr int kTileBytes = kBoxBytes * kBoxes;
   static constexpr int kKStages = (D == 128) ? 3 : 4;
-  static constexpr int kVStages = (D == 128) ? 2 : 4;
+  static constexpr int kVStages = (D == 128) ? 2 : 6;
   static constexpr int kOffQ0 = 0;
   static constexpr int kOffQ1 = kTileBytes;
   static constexpr int kOffK = 2 * kTileBytes;
   static constexpr int kOffV = kOffK + kKStages * kTileBytes;
   static constexpr int kSmemBytes = kOffV + kVStages * kTileBytes + 1024;  // + alignment slack
   static constexpr uint32_t kTmemCols = 512;
+  // Head dimension 64: each softmax warpgroup owns one query tile (a thread
+  // per row), three S buffers.  See the note above the kernel.
+  static constexpr bool kOwnTile = D == 64;
+  static constexpr int kStepBars = kOwnTile ? 6 : 2;        // S (and P) barriers
+  static constexpr int kTilesPerWarp = kOwnTile ? 1 : 2;    // query tiles a softmax warp works on
+  static constexpr int kRowThreads = kOwnTile ? 1 : 2;      // threads per query row
+  static constexpr int kChunks = 4 / kRowThreads;           // 32-key chunks of a row per thread
 };
 
-// TMEM columns of the S buffers and O accumulators of query tiles 0 and 1.
-__device__ __forceinline__ uint32_t col_s(int b) { return b ? 128u : 0u; }
-__device__ __forceinline__ uint32_t col_o(int b) { return b ? 384u : 256u; }
+// TMEM columns.  D = 128: one S buffer per query tile and the two O
+// accumulators fill the 512 columns.  D = 64: O takes 64 columns a tile, which
+// leaves room for a third S buffer; the steps (key tile, query tile) take the
+// three in turn.
+template <int D>
+__device__ __forceinline__ uint32_t col_s(int buf) {
+  return (uint32_t)buf * 128u;
+}
+template <int D>
+__device__ __forceinline__ uint32_t col_o(int b) {
+  return D == 128 ? (b ? 384u : 256u) : (b ? 448u : 384u);
+}
 
 // 12 warps: warpgroup 0 = TMA producer (warp 0), MMA issuers (warps 1 and
 // 3), warp 2 (the block-sparse mask gather in the prologue, then idle);
@@ -148,14 +186,18 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 
 struct Bars {
   uint64_t q_full;
-  uint64_t s_full[2];
-  uint64_t p_full[2];
+  // S and P of a query tile's steps.  D = 128: one each per query tile.  D =
+  // 64: three per query tile taken in turn, so that each barrier has one
+  // waiter, which waits for every phase (the S of a query tile run up to two
+  // key tiles ahead of its softmax, and its P up to two ahead of the issuer).
+  uint64_t s_full[6];
+  uint64_t p_full[6];
   uint64_t o_final;
   uint64_t drain;
   uint64_t k_full[4];
   uint64_t k_empty[4];
-  uint64_t v_full[4];
-  uint64_t v_empty[4];
+  uint64_t v_full[6];
+  uint64_t v_empty[6];
 };
 
 // Block-sparse launches: a role's walk over the key tiles that either query
@@ -255,17 +297,17 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     mbar_init(&bars.q_full, 1);
     mbar_init(&bars.o_final, 2);  // one commit per MMA issuer
     mbar_init(&bars.drain, 2);
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < C::kStepBars; ++b) {
       mbar_init(&bars.s_full[b], 1);
-      mbar_init(&bars.p_full[b], 256);
+      mbar_init(&bars.p_full[b], 128 * C::kRowThreads);
     }
     for (int s = 0; s < C::kKStages; ++s) {
       mbar_init(&bars.k_full[s], 1);
-      mbar_init(&bars.k_empty[s], 1);
+      mbar_init(&bars.k_empty[s], C::kOwnTile && has_q1 ? 2 : 1);  // D = 64: one per query tile
     }
     for (int s = 0; s < C::kVStages; ++s) {
       mbar_init(&bars.v_full[s], 1);
-      mbar_init(&bars.v_empty[s], 1);
+      mbar_init(&bars.v_empty[s], C::kOwnTile && has_q1 ? 2 : 1);
     }
     fence_mbar_init();
   }
@@ -414,26 +456,33 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         return !sparse || ((tmask[b][kt >> 5] >> (kt & 31)) & 1u) != 0u;
       };
       bool pv_started = false;  // this issuer's query tile has a PV in O
-      // S_b = Q_b K_i^T into TMEM buffer b
-      auto issue_s = [&](int b, int i, bool v) {
+      // S_b = Q_b K_i^T into TMEM buffer `buf`, then a commit to S barrier `bar`
+      auto issue_s = [&](int b, int buf, int bar, int i, bool v) {
         if (v) {
           const uint64_t kb = dK + (uint64_t)(i % C::kKStages) * kTileStep;
           const uint64_t qb = b == 0 ? dQ[0] : dQ[1];
-          const uint32_t dcol = tbase + col_s(b);
+          const uint32_t dcol = tbase + col_s<D>(buf);
+          if constexpr (C::kOwnTile) {
+            mma_ss_warp_x4(dcol, qb, kb, 2, idesc_qk);
+          } else {
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint64_t off = (uint64_t)(((kk >> 2) * C::kBoxBytes + (kk & 3) * 32) >> 4);
-            mma_ss_warp(dcol, qb + off, kb + off, idesc_qk, kk > 0 ? 1u : 0u);
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint64_t off = (uint64_t)(((kk >> 2) * C::kBoxBytes + (kk & 3) * 32) >> 4);
+              mma_ss_warp(dcol, qb + off, kb + off, idesc_qk, kk > 0 ? 1u : 0u);
+            }
           }
         }
-        mma_commit_warp(&bars.s_full[b]);
+        mma_commit_warp(&bars.s_full[bar]);
       };
-      // O_b += P_b V_i with P_b read from TMEM over S_b
-      auto issue_pv = [&](int b, int i) {
+      // O_b += P_b V_i with P_b read from TMEM over S_b in buffer `buf`
+      auto issue_pv = [&](int b, int buf, int i) {
         const uint64_t vb = dV + (uint64_t)(i % C::kVStages) * kTileStep;
-        const uint32_t ocol = tbase + col_o(b);
-        const uint32_t pcol = tbase + col_s(b);
+        const uint32_t ocol = tbase + col_o<D>(b);
+        const uint32_t pcol = tbase + col_s<D>(buf);
         const uint32_t acc0 = (sparse ? pv_started : i > 0) ? 1u : 0u;
+        if constexpr (C::kOwnTile)
+          mma_ts_warp_x8(ocol, pcol, vb, idesc_pv, acc0);
+        else
 #pragma unroll
         for (int kk = 0; kk < kTile / 16; ++kk)
           mma_ts_warp(ocol, pcol + kk * 8, vb + (uint64_t)((kk * 2048) >> 4), idesc_pv,
@@ -446,9 +495,74 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       auto wait_k = [&](int i) {
         return wait(&bars.k_full[i % C::kKStages], (uint32_t)(i / C::kKStages) & 1u);
       };
-      const int bq = warp == 1 ? 0 : 1;  // the query tile this warp issues for
+      const int bq = warp == 1 ? 0 : 1;  // the query tile this warp issues for (D = 128)
       bool ok = wait(&bars.q_full, 0);
-      if (bq == 0 || has_q1) {
+      if constexpr (C::kOwnTile) {
+        // Steps n = (key tile i, query tile b), b fastest, in S buffer n % 3:
+        // when P_n is there, PV_n is issued and right behind it S_{n+3}, which
+        // overwrites the buffer that PV_n reads (the MMAs of one thread
+        // execute in issue order).  Two issuers: warp 1 takes the even n (PV
+        // of query tile 0, S of query tile 1), warp 3 the odd n (PV of query
+        // tile 1, S of query tile 0).  With one query tile warp 1 takes all.
+        const int nb = has_q1 ? 2 : 1;
+        if (bq < nb) {
+          const int qs = nb - 1 - bq;  // the query tile whose S this warp issues
+          TileWalk<kSparse ? kMaskWords : 1> walk_s, walk_p;
+          if constexpr (sparse) {
+            walk_s.start(tmask, t_begin, n_all);
+            walk_p.start(tmask, t_begin, n_all);
+          }
+          int si = 0, skt = 0;  // tile of the next S and its key tile of the node
+          auto next_kt_s = [&]() {
+            if constexpr (sparse) skt = walk_s.next();
+          };
+          // ahead: S steps issued before the first PV (of the first three steps)
+          const int ahead = nb == 1 ? 3 : 1 + bq;
+          for (int k = 0; ok && k < ahead && si < n_tiles; ++k, ++si) {
+            next_kt_s();
+            ok = wait_k(si);
+            if (!ok) break;
+            tc_fence_after();
+            issue_s(qs, nb == 1 ? k : qs + 2 * k, qs * 3 + k, si, vis(qs, skt));
+          }
+          int buf = bq;             // S buffer of step n = nb * i + bq
+          int bar = 0;              // i % 3 and the phase of that P barrier
+          uint32_t par = 0;
+          for (int i = 0; ok && i < n_tiles; ++i) {
+            const bool more = si < n_tiles;
+            int pkt = 0;
+            if constexpr (sparse) pkt = walk_p.next();
+            if (more) next_kt_s();
+            // V_i and the next S's K normally landed long ago: one round trip
+            // tests both
+            uint64_t* vbar = &bars.v_full[i % C::kVStages];
+            uint64_t* kbar = &bars.k_full[more ? si % C::kKStages : 0];
+            const uint32_t vpar = (uint32_t)(i / C::kVStages) & 1u;
+            const uint32_t kpar = (uint32_t)(si / C::kKStages) & 1u;
+            const bool vok = mbar_try_wait(vbar, vpar);
+            const bool kok = !more || mbar_try_wait(kbar, kpar);
+            if (!__all_sync(0xffffffffu, vok && kok))
+              ok = wait(vbar, vpar) && (!more || wait(kbar, kpar));
+            if (!ok || !wait(&bars.p_full[bq * 3 + bar], par)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            if (vis(bq, pkt)) issue_pv(bq, buf, i);
+            mma_commit_warp(&bars.v_empty[i % C::kVStages]);
+            if (more) {
+              issue_s(qs, buf, qs * 3 + si % 3, si, vis(qs, skt));
+              ++si;
+            }
+            buf += nb;
+            if (buf >= 3) buf -= 3;
+            if (++bar == 3) {
+              bar = 0;
+              par ^= 1u;
+            }
+          }
+        }
+      } else if (bq == 0 || has_q1) {
         TileWalk<kSparse ? kMaskWords : 1> walk;
         if constexpr (sparse) walk.start(tmask, t_begin, n_all);
         int kt = sparse ? walk.next() : t_begin;  // key tile of the node at iteration i
@@ -456,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           ok = ok && wait_k(0);
           if (ok) {
             tc_fence_after();
-            issue_s(bq, 0, vis(bq, kt));
+            issue_s(bq, bq, bq, 0, vis(bq, kt));
           }
         }
         for (int i = 0; ok && i < n_tiles; ++i) {
@@ -472,8 +586,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
             break;
           }
           tc_fence_after();
-          if (vis_cur) issue_pv(bq, i);
-          if (more) issue_s(bq, i + 1, vis_next);
+          if (vis_cur) issue_pv(bq, bq, i);
+          if (more) issue_s(bq, bq, bq, i + 1, vis_next);
           kt = kt_next;
         }
       }
@@ -515,122 +629,148 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   } else {
     regs_inc<kRegsHigh>();
     // ------------------------------------------------------------ softmax + epilogue
-    // All eight softmax warps work on one query tile at a time (tile 0, then
-    // tile 1, of every key tile).  A warp covers 16 rows, half of its TMEM
-    // lane quarter, with two threads per row (16x32bx2 shape): thread t < 16
-    // holds keys 0..63 of its row, thread t + 16 keys 64..127 of the same
+    // D = 128: all eight softmax warps work on one query tile at a time (tile
+    // 0, then tile 1, of every key tile).  A warp covers 16 rows, half of its
+    // TMEM lane quarter, with two threads per row (16x32bx2 shape): thread t <
+    // 16 holds keys 0..63 of its row, thread t + 16 keys 64..127 of the same
     // row.  Both threads of a row keep the same running max (the two halves'
     // maxima are exchanged with one shuffle) and each its part of the sum,
     // so each thread exponentiates 64 keys per tile instead of 128 and the
     // two warps sharing a sub-partition overlap their MUFU and FMA work.
-    constexpr int DH = D / 2;                      // output columns per thread
+    // D = 64: warps 4-7 take query tile 0, warps 8-11 tile 1, a thread per row
+    // with all 128 keys; see the note above the kernel.
+    constexpr int NT = C::kTilesPerWarp;           // query tiles this warp works on
+    constexpr int NC = C::kChunks;                 // 32-key chunks per thread
+    constexpr int DH = D / C::kRowThreads;         // output columns per thread
     const int q4 = warp & 3;                       // TMEM lane quarter this warp may access
-    const int hi = warp >> 3;                      // which 16 lanes of the quarter
-    const int half = lane >> 4;                    // which 64 keys, which D/2 columns
-    const int row = q4 * 32 + hi * 16 + (lane & 15);  // query row inside a tile
-    const uint32_t lane_off = (uint32_t)(q4 * 32 + hi * 16) << 16;
+    const int hi = warp >> 3;                      // D = 128: which 16 lanes of the quarter
+    const int half = C::kOwnTile ? 0 : lane >> 4;  // which 64 keys, which D/2 columns
+    // query row inside a tile, and the warp's first TMEM lane
+    const int row = C::kOwnTile ? q4 * 32 + lane : q4 * 32 + hi * 16 + (lane & 15);
+    const uint32_t lane_off = (uint32_t)(C::kOwnTile ? q4 * 32 : q4 * 32 + hi * 16) << 16;
+    const int b_own = hi;                          // D = 64: this warpgroup's query tile
     const int nb = has_q1 ? 2 : 1;
     const float sl2 = p.scale_log2;
     const uint64_t sl2x2 = f2u(sl2, sl2);
     const int frame_causal = nd.frame_causal;
-    bool o_has[2] = {false, false};       // O_b holds a PV (some key tile was attended)
-    float m[2] = {-INFINITY, -INFINITY};  // running max of scale*log2(e)*logit per query tile
-    float l[2] = {0.0f, 0.0f};            // this thread's part of the running sum of 2^(x - m)
-    // first token of the latent frame after this row's (frame-causal mask)
-    int frame_end[2];
+    // 32 output columns of this thread's row in O, from TMEM and back
+    auto ld_o = [&](uint32_t col, uint32_t (&o)[32]) {
+      if constexpr (C::kOwnTile)
+        tmem_ld32(tbase + lane_off + col, o);
+      else
+        tmem_ld16x2_32<DH>(tbase + lane_off + col, o);
+      tmem_wait_ld(o);
+    };
+    auto st_o = [&](uint32_t col, const uint32_t (&o)[32]) {
+      if constexpr (C::kOwnTile)
+        tmem_st32(tbase + lane_off + col, o);
+      else
+        tmem_st16x2_32<DH>(tbase + lane_off + col, o);
+    };
+    bool o_has[NT];       // O_b holds a PV (some key tile was attended)
+    float m[NT];          // running max of scale*log2(e)*logit per query tile
+    float l[NT];          // this thread's part of the running sum of 2^(x - m)
+    int frame_end[NT];    // first token of the latent frame after this row's (frame-causal mask)
 #pragma unroll
-    for (int b = 0; b < 2; ++b)
-      frame_end[b] = ((qt0 + b) * kTile + row) / p.frame_tokens * p.frame_tokens + p.frame_tokens;
-    // The softmax sees S_0 and then S_1 of key tile i complete.  S_b,i
-    // follows PV_b,i-1 in its issuer's order, so once both are seen every
+    for (int x = 0; x < NT; ++x) {
+      const int b = C::kOwnTile ? b_own : x;
+      o_has[x] = false;
+      m[x] = -INFINITY;
+      l[x] = 0.0f;
+      frame_end[x] = ((qt0 + b) * kTile + row) / p.frame_tokens * p.frame_tokens + p.frame_tokens;
+    }
+    // D = 128: the softmax sees S_0 and then S_1 of key tile i complete.
+    // S_b,i follows PV_b,i-1 in its issuer's order, so once both are seen every
     // MMA that reads K stage i or V stage i-1 has completed, and one softmax
     // thread hands both stages back to the producer when it sees the last S
     // of the tile (S_1, or S_0 without a second query tile).  The MMA warps
     // then commit only to their S barriers (a commit costs an issuer about
-    // as long as an MMA).
-    const bool releaser = warp == 4 && lane == 0;
+    // as long as an MMA).  D = 64: one thread per query tile hands back K
+    // stage i when it sees S_b,i; the issuers' commits hand back the V stages.
+    const bool releaser = (C::kOwnTile ? q4 == 0 : warp == 4) && lane == 0;
     bool ok = true;
     TileWalk<kSparse ? kMaskWords : 1> walk;
     if constexpr (sparse) walk.start(tmask, t_begin, n_all);
     int kt = sparse ? walk.next() : t_begin;  // key tile of the node
-    int kt_next = kt;
-    for (int i = 0; ok && i < n_tiles; ++i, kt = kt_next) {
-      // The next tile of the walk and, under a tile mask, which query tiles
-      // attend this one: read from shared memory before the S wait, so their
-      // latency is not added to the path from S to P.
-      kt_next = sparse ? walk.next() : next_kt(kt);
-      const uint32_t attends = sparse ? ((tmask[0][kt >> 5] >> (kt & 31)) & 1u) |
-                                            (((tmask[1][kt >> 5] >> (kt & 31)) & 1u) << 1)
-                                      : 3u;
-      const int t = kt % p.nt_slot;  // key tile inside its slot
-      const int valid_tile = (t == p.nt_slot - 1) ? p.valid_last : kTile;
-      const bool own_fc = frame_causal && kt < p.nt_slot;
+    if constexpr (C::kOwnTile) {
+      const int b = b_own;
+      int kst = kt / p.nt_slot;                 // its key state: 0 own, then the visible contexts
+      int t = kt - kst * p.nt_slot;             // and its place in the state's slot
+      // Steps to the next key tile of the walk.  A dense walk visits the tiles
+      // of a slot in order (with the frame-causal gap at the end of the own
+      // slot), so no division is needed; a block-sparse one divides by a
+      // reciprocal (exact: kt < 2^12 and nt_slot <= 2^9).
+      const uint32_t inv_nt = p.nt_slot > 1 ? 0xFFFFFFFFu / (uint32_t)p.nt_slot + 1u : 0u;
+      auto advance = [&](int next) {
+        if constexpr (sparse) {
+          kst = inv_nt ? (int)__umulhi((uint32_t)next, inv_nt) : next;
+          t = next - kst * p.nt_slot;
+        } else {
+          t += next - kt;
+          if (t >= p.nt_slot) {  // also from a tile before the gap to the next slot's first
+            t = 0;
+            ++kst;
+          }
+        }
+        kt = next;
+      };
+      auto attends = [&](int tile) {
+        return !sparse || ((tmask[b][tile >> 5] >> (tile & 31)) & 1u) != 0u;
+      };
+      auto wait_s = [&](int bar, uint32_t par) {
+        return __all_sync(0xffffffffu, mbar_wait(&bars.s_full[b * 3 + bar], par, &abort_flag, tmo)) != 0;
+      };
+      // token-level mask (token-mask instance): this thread's bits of its row
+      // for the key tile, from the own-chunk mask or from the history mask of
+      // the tile's key state (the caller's context index)
+      auto token_bits = [&](uint32_t (&ow)[NC]) {
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        if (b == 1 && !has_q1) break;
-        // token-level mask (token-mask instance): this thread's 64 bits of its
-        // row for this key tile, from the own-chunk mask or from the history
-        // mask of the tile's key state (the caller's context index); fetched
-        // before the wait so that the load hides behind it
-        const int kst = kOwn ? kt / p.nt_slot : 0;  // key state: 0 own, then the visible contexts
-        const bool own_tile = kOwn && (kst == 0 ? p.own_mask : p.hist_mask) != nullptr;
-        uint32_t ow[2] = {~0u, ~0u};
-        if (own_tile) {
+        for (int c = 0; c < NC; ++c) ow[c] = ~0u;
+        if constexpr (kOwn) {
+          const bool masked = (kst == 0 ? p.own_mask : p.hist_mask) != nullptr;
           const int u = (qt0 + b) * kTile + row;
-          if (u < p.T) {  // rows past T are never stored
+          if (masked && u < p.T) {  // rows past T are never stored
             const size_t qrow = (size_t)nd.q_index * p.T + u;
             const uint32_t* mrow =
                 kst == 0 ? p.own_mask + qrow * p.own_words
                          : p.hist_mask + (qrow * p.hist_states + (nd.src[kst] - 1)) * p.hist_words;
             const int words = kst == 0 ? p.own_words : p.hist_words;
-            const int wi = (kt - kst * p.nt_slot) * 4 + half * 2;  // key 128 t + 64 half of the state
-            ow[0] = wi < words ? __ldg(mrow + wi) : 0u;
-            ow[1] = wi + 1 < words ? __ldg(mrow + wi + 1) : 0u;
+            const int wi = t * 4;  // key 128 t of the state
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ow[c] = wi + c < words ? __ldg(mrow + wi + c) : 0u;
           }
+          return masked;
         }
-        ok = mbar_wait(&bars.s_full[b], (uint32_t)i & 1u, &abort_flag, tmo);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        if (releaser && b == nb - 1) {
-          mbar_arrive(&bars.k_empty[i % C::kKStages]);
-          if (i > 0) mbar_arrive(&bars.v_empty[(i - 1) % C::kVStages]);
-        }
-        if (sparse && !((attends >> b) & 1u)) {
-          // query tile b skips this key tile: no S was computed, no P is due
-          mbar_arrive(&bars.p_full[b]);
-          continue;
-        }
-        tc_fence_after();
-        const uint32_t scol = tbase + lane_off + col_s(b);
-        const uint32_t ocol = tbase + lane_off + col_o(b);
-        // own-chunk tile under frame causality: keys up to the end of this
-        // row's latent frame are visible (tile 0, frame 0, always is)
-        const int valid = own_fc ? min(valid_tile, frame_end[b] - t * kTile) : valid_tile;
-        const int vrel = valid - half * 64;  // visible keys among this thread's 64
-        // The loads also reduce each 32-column chunk to its maximum, so a
-        // full tile needs no max tree; a tile with masked keys (the ragged
-        // last tile of a slot, frame causality) takes the max over what is
-        // left after masking.
-        uint32_t s[2][32];
-        float cmax[2];
-        tmem_ld16x2_32_max<64>(scol, s[0], cmax[0]);
-        tmem_ld16x2_32_max<64>(scol + 32, s[1], cmax[1]);
-        tmem_wait_ld(s[0]);
-        tmem_wait_ld(s[1]);
-        tmem_wait_ld_max2(cmax);
-        float m_part = fmaxf(cmax[0], cmax[1]);
-        // Tiles that can hold masked keys (a slot's ragged last tile, the own
-        // chunk under frame causality) take the masked path; the test is the
-        // same for every thread, so it needs no vote.
+        return false;
+      };
+      // One step from its scores s (with the maximum cmax of each 32-key chunk)
+      // up to the row's running max: masks, then moves m and rescales O and l
+      // where a row needs it.  False: a wait expired.
+      auto row_max = [&](int i, uint32_t (&s)[NC][32], const float (&cmax)[NC],
+                         const uint32_t (&ow)[NC], bool own_tile) {
+        float m_part = cmax[0];
+#pragma unroll
+        for (int c = 1; c < NC; ++c) m_part = fmaxf(m_part, cmax[c]);
+        const int valid_tile = (t == p.nt_slot - 1) ? p.valid_last : kTile;
+        const bool own_fc = frame_causal && kst == 0;
+        // The loads also reduce each 32-column chunk to its maximum, so a full
+        // tile needs no max tree; tiles that can hold masked keys (a slot's
+        // ragged last tile, the own chunk under frame causality) take the max
+        // over what is left after masking.  The test is the same for every
+        // thread, so it needs no vote.
         if (valid_tile < kTile || own_fc || own_tile) {
+          // own-chunk tile under frame causality: keys up to the end of this
+          // row's latent frame are visible (tile 0, frame 0, always is)
+          const int valid = own_fc ? min(valid_tile, frame_end[0] - t * kTile) : valid_tile;
+          const int vrel = valid;
           float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-          for (int c = 0; c < 2; ++c)
+          for (int c = 0; c < NC; ++c)
 #pragma unroll
             for (int e = 0; e < 32; ++e)
               if (c * 32 + e >= vrel || !((ow[c] >> e) & 1u)) s[c][e] = __float_as_uint(-INFINITY);
 #pragma unroll
-          for (int c = 0; c < 2; ++c)
+          for (int c = 0; c < NC; ++c)
 #pragma unroll
             for (int e = 0; e < 32; e += 8) {
               const int k = (c & 1) * 2 + (e >> 4);
@@ -641,64 +781,259 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
             }
           m_part = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
         }
-        const float m_tile = fmaxf(m_part, __shfl_xor_sync(0xffffffffu, m_part, 16)) * sl2;
-        const float m_new = fmaxf(m[b], m_tile);
-        const bool need = m_new > m[b] + kRescaleThreshold;
+        const float m_tile = m_part * sl2;
+        const float m_new = fmaxf(m[0], m_tile);
+        const bool need = m_new > m[0] + kRescaleThreshold;
         if (__any_sync(0xffffffffu, need)) {
           // 0 when the row's first visible keys arrive (m = -inf); 1 for a row
           // of the warp whose max did not move (also when it is still -inf:
           // -inf - -inf would be NaN)
-          const float alpha = m_new > m[b] ? ex2(m[b] - m_new) : 1.0f;
-          if (sparse ? o_has[b] : i > 0) {
-            // O_b holds the sum over earlier tiles: the commit that completed
-            // S_b of this tile came after PV_b of the previous one.
+          const float alpha = m_new > m[0] ? ex2(m[0] - m_new) : 1.0f;
+          if (sparse ? o_has[0] : i > 0) {
+            // O_b holds the sum over earlier tiles.  S runs ahead of the PVs, so
+            // the commit that follows PV of the previous tile and frees its V
+            // stage is waited for (that stage's next phase cannot end before
+            // this step's PV).
+            const bool pv = mbar_wait(&bars.v_empty[(i - 1) % C::kVStages],
+                                      (uint32_t)((i - 1) / C::kVStages) & 1u, &abort_flag, tmo);
+            if (!__all_sync(0xffffffffu, pv)) return false;
+            tc_fence_after();
 #pragma unroll
             for (int c = 0; c < DH / 32; ++c) {
               uint32_t o[32];
-              tmem_ld16x2_32<DH>(ocol + c * 32, o);
-              tmem_wait_ld(o);
+              ld_o(col_o<D>(b) + c * 32, o);
 #pragma unroll
               for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-              tmem_st16x2_32<DH>(ocol + c * 32, o);
+              st_o(col_o<D>(b) + c * 32, o);
             }
             tmem_wait_st();
           }
-          l[b] *= alpha;
-          m[b] = m_new;
+          l[0] *= alpha;
+          m[0] = m_new;
         }
-        // m stays -inf while a row has seen no visible key (possible in a key
-        // range that starts past a row's frame under frame causality); its
-        // scores are then all -inf and must give P = 0, not NaN.
-        const float m_sub = (m[b] == -INFINITY) ? 0.0f : m[b];
-        const uint64_t negm = f2u(-m_sub, -m_sub);
-        uint64_t acc[4] = {0, 0, 0, 0};
-        // P of 32 keys packs into 16 words, written over the first half of
-        // the same registers (word e/2 is written after elements e, e+1 are
-        // read); the two halves make one 32-column store over S (keys
-        // 0..63 of the row at columns 0..31, keys 64..127 at 32..63).
+        return true;
+      };
+      // P of a chunk of 32 keys, packed into the first 16 registers of its
+      // scores (word e/2 is written after elements e, e+1 are read), and its
+      // part of the row sum.  m stays -inf while a row has seen no visible key
+      // (possible in a key range that starts past a row's frame under frame
+      // causality); its scores are then all -inf and must give P = 0, not NaN.
+      auto expo = [&](uint32_t (&sc)[32], uint64_t negm, uint64_t (&acc)[4]) {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            float x0, x1;
-            ffma2(x0, x1, __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]), sl2x2, negm);
-            const float p0 = ex2(x0);
-            const float p1 = ex2(x1);
-            acc[(e >> 1) & 3] = fadd2(acc[(e >> 1) & 3], p0, p1);
-            s[c][e >> 1] = pack_bf16(p0, p1);
-          }
+        for (int e = 0; e < 32; e += 2) {
+          float x0, x1;
+          ffma2(x0, x1, __uint_as_float(sc[e]), __uint_as_float(sc[e + 1]), sl2x2, negm);
+          const float p0 = ex2(x0);
+          const float p1 = ex2(x1);
+          acc[(e >> 1) & 3] = fadd2(acc[(e >> 1) & 3], p0, p1);
+          sc[e >> 1] = pack_bf16(p0, p1);
         }
-        tmem_st16x2_32_halves<32>(scol, s[0], s[1]);
+      };
+      auto neg_max = [&]() {
+        const float m_sub = (m[0] == -INFINITY) ? 0.0f : m[0];
+        return f2u(-m_sub, -m_sub);
+      };
+      auto add_sum = [&](const uint64_t (&acc)[4]) {
         float a0, a1, a2, a3, a4, a5, a6, a7;
         u2f(acc[0], a0, a1);
         u2f(acc[1], a2, a3);
         u2f(acc[2], a4, a5);
         u2f(acc[3], a6, a7);
-        l[b] += ((a0 + a1) + (a2 + a3)) + ((a4 + a5) + (a6 + a7));
-        tmem_wait_st();
-        tc_fence_before();
-        mbar_arrive(&bars.p_full[b]);
-        if (sparse) o_has[b] = true;
+        l[0] += ((a0 + a1) + (a2 + a3)) + ((a4 + a5) + (a6 + a7));
+      };
+      const int my_tiles = b < nb ? n_tiles : 0;
+      int buf = b, bar = 0;  // S buffer of step n = nb * i + b; i % 3 and that barrier's phase
+      uint32_t par = 0;
+      for (int i = 0; ok && i < my_tiles; ++i) {
+        const int kt_next = sparse ? walk.next() : next_kt(kt);
+        uint64_t* p_bar = &bars.p_full[b * 3 + bar];
+        ok = wait_s(bar, par);
+        if (!ok) break;
+        if (releaser) mbar_arrive(&bars.k_empty[i % C::kKStages]);
+        if (attends(kt)) {  // else no S was computed and no P is due
+          tc_fence_after();
+          const uint32_t scol = tbase + lane_off + col_s<D>(buf);
+          uint32_t s[NC][32];
+          float cmax[NC];
+#pragma unroll
+          for (int c = 0; c < NC; ++c) tmem_ld32_max(scol + c * 32, s[c], cmax[c]);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) tmem_wait_ld(s[c]);
+          tmem_wait_ld_max(cmax);
+          uint32_t ow[NC];
+          const bool own_tile = token_bits(ow);
+          ok = row_max(i, s, cmax, ow, own_tile);
+          if (!ok) break;
+          const uint64_t negm = neg_max();
+          uint64_t acc[4] = {0, 0, 0, 0};
+          expo(s[0], negm, acc);
+          expo(s[1], negm, acc);
+          tmem_st32_halves(scol, s[0], s[1]);
+          expo(s[2], negm, acc);
+          expo(s[3], negm, acc);
+          tmem_st32_halves(scol + 32, s[2], s[3]);
+          tmem_wait_st();
+          tc_fence_before();
+          add_sum(acc);
+          o_has[0] = true;
+        }
+        mbar_arrive(p_bar);
+        advance(kt_next);
+        buf += nb;
+        if (buf >= 3) buf -= 3;
+        if (++bar == 3) {
+          bar = 0;
+          par ^= 1u;
+        }
+      }
+    } else {
+      int kt_next = kt;
+      for (int i = 0; ok && i < n_tiles; ++i, kt = kt_next) {
+        // The next tile of the walk and, under a tile mask, which query tiles
+        // attend this one: read from shared memory before the S wait, so their
+        // latency is not added to the path from S to P.
+        kt_next = sparse ? walk.next() : next_kt(kt);
+        const uint32_t attends = sparse ? ((tmask[0][kt >> 5] >> (kt & 31)) & 1u) |
+                                              (((tmask[1][kt >> 5] >> (kt & 31)) & 1u) << 1)
+                                        : 3u;
+        const int t = kt % p.nt_slot;  // key tile inside its slot
+        const int valid_tile = (t == p.nt_slot - 1) ? p.valid_last : kTile;
+        const bool own_fc = frame_causal && kt < p.nt_slot;
+  #pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          if (b == 1 && !has_q1) break;
+          // token-level mask (token-mask instance): this thread's 64 bits of its
+          // row for this key tile, from the own-chunk mask or from the history
+          // mask of the tile's key state (the caller's context index); fetched
+          // before the wait so that the load hides behind it
+          const int kst = kOwn ? kt / p.nt_slot : 0;  // key state: 0 own, then the visible contexts
+          const bool own_tile = kOwn && (kst == 0 ? p.own_mask : p.hist_mask) != nullptr;
+          uint32_t ow[2] = {~0u, ~0u};
+          if (own_tile) {
+            const int u = (qt0 + b) * kTile + row;
+            if (u < p.T) {  // rows past T are never stored
+              const size_t qrow = (size_t)nd.q_index * p.T + u;
+              const uint32_t* mrow =
+                  kst == 0 ? p.own_mask + qrow * p.own_words
+                           : p.hist_mask + (qrow * p.hist_states + (nd.src[kst] - 1)) * p.hist_words;
+              const int words = kst == 0 ? p.own_words : p.hist_words;
+              const int wi = (kt - kst * p.nt_slot) * 4 + half * 2;  // key 128 t + 64 half of the state
+              ow[0] = wi < words ? __ldg(mrow + wi) : 0u;
+              ow[1] = wi + 1 < words ? __ldg(mrow + wi + 1) : 0u;
+            }
+          }
+          ok = mbar_wait(&bars.s_full[b], (uint32_t)i & 1u, &abort_flag, tmo);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          if (releaser && b == nb - 1) {
+            mbar_arrive(&bars.k_empty[i % C::kKStages]);
+            if (i > 0) mbar_arrive(&bars.v_empty[(i - 1) % C::kVStages]);
+          }
+          if (sparse && !((attends >> b) & 1u)) {
+            // query tile b skips this key tile: no S was computed, no P is due
+            mbar_arrive(&bars.p_full[b]);
+            continue;
+          }
+          tc_fence_after();
+          const uint32_t scol = tbase + lane_off + col_s<D>(b);
+          const uint32_t ocol = tbase + lane_off + col_o<D>(b);
+          // own-chunk tile under frame causality: keys up to the end of this
+          // row's latent frame are visible (tile 0, frame 0, always is)
+          const int valid = own_fc ? min(valid_tile, frame_end[b] - t * kTile) : valid_tile;
+          const int vrel = valid - half * 64;  // visible keys among this thread's 64
+          // The loads also reduce each 32-column chunk to its maximum, so a
+          // full tile needs no max tree; a tile with masked keys (the ragged
+          // last tile of a slot, frame causality) takes the max over what is
+          // left after masking.
+          uint32_t s[2][32];
+          float cmax[2];
+          tmem_ld16x2_32_max<64>(scol, s[0], cmax[0]);
+          tmem_ld16x2_32_max<64>(scol + 32, s[1], cmax[1]);
+          tmem_wait_ld(s[0]);
+          tmem_wait_ld(s[1]);
+          tmem_wait_ld_max2(cmax);
+          float m_part = fmaxf(cmax[0], cmax[1]);
+          // Tiles that can hold masked keys (a slot's ragged last tile, the own
+          // chunk under frame causality) take the masked path; the test is the
+          // same for every thread, so it needs no vote.
+          if (valid_tile < kTile || own_fc || own_tile) {
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  #pragma unroll
+            for (int c = 0; c < 2; ++c)
+  #pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (c * 32 + e >= vrel || !((ow[c] >> e) & 1u)) s[c][e] = __float_as_uint(-INFINITY);
+  #pragma unroll
+            for (int c = 0; c < 2; ++c)
+  #pragma unroll
+              for (int e = 0; e < 32; e += 8) {
+                const int k = (c & 1) * 2 + (e >> 4);
+                mx[k] = max3(mx[k], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
+                mx[k] = max3(mx[k], __uint_as_float(s[c][e + 2]), __uint_as_float(s[c][e + 3]));
+                mx[k] = max3(mx[k], __uint_as_float(s[c][e + 4]), __uint_as_float(s[c][e + 5]));
+                mx[k] = max3(mx[k], __uint_as_float(s[c][e + 6]), __uint_as_float(s[c][e + 7]));
+              }
+            m_part = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          }
+          const float m_tile = fmaxf(m_part, __shfl_xor_sync(0xffffffffu, m_part, 16)) * sl2;
+          const float m_new = fmaxf(m[b], m_tile);
+          const bool need = m_new > m[b] + kRescaleThreshold;
+          if (__any_sync(0xffffffffu, need)) {
+            // 0 when the row's first visible keys arrive (m = -inf); 1 for a row
+            // of the warp whose max did not move (also when it is still -inf:
+            // -inf - -inf would be NaN)
+            const float alpha = m_new > m[b] ? ex2(m[b] - m_new) : 1.0f;
+            if (sparse ? o_has[b] : i > 0) {
+              // O_b holds the sum over earlier tiles: the commit that completed
+              // S_b of this tile came after PV_b of the previous one.
+  #pragma unroll
+              for (int c = 0; c < DH / 32; ++c) {
+                uint32_t o[32];
+                tmem_ld16x2_32<DH>(ocol + c * 32, o);
+                tmem_wait_ld(o);
+  #pragma unroll
+                for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                tmem_st16x2_32<DH>(ocol + c * 32, o);
+              }
+              tmem_wait_st();
+            }
+            l[b] *= alpha;
+            m[b] = m_new;
+          }
+          // m stays -inf while a row has seen no visible key (possible in a key
+          // range that starts past a row's frame under frame causality); its
+          // scores are then all -inf and must give P = 0, not NaN.
+          const float m_sub = (m[b] == -INFINITY) ? 0.0f : m[b];
+          const uint64_t negm = f2u(-m_sub, -m_sub);
+          uint64_t acc[4] = {0, 0, 0, 0};
+          // P of 32 keys packs into 16 words, written over the first half of
+          // the same registers (word e/2 is written after elements e, e+1 are
+          // read); the two halves make one 32-column store over S (keys
+          // 0..63 of the row at columns 0..31, keys 64..127 at 32..63).
+  #pragma unroll
+          for (int c = 0; c < 2; ++c) {
+  #pragma unroll
+            for (int e = 0; e < 32; e += 2) {
+              float x0, x1;
+              ffma2(x0, x1, __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]), sl2x2, negm);
+              const float p0 = ex2(x0);
+              const float p1 = ex2(x1);
+              acc[(e >> 1) & 3] = fadd2(acc[(e >> 1) & 3], p0, p1);
+              s[c][e >> 1] = pack_bf16(p0, p1);
+            }
+          }
+          tmem_st16x2_32_halves<32>(scol, s[0], s[1]);
+          float a0, a1, a2, a3, a4, a5, a6, a7;
+          u2f(acc[0], a0, a1);
+          u2f(acc[1], a2, a3);
+          u2f(acc[2], a4, a5);
+          u2f(acc[3], a6, a7);
+          l[b] += ((a0 + a1) + (a2 + a3)) + ((a4 + a5) + (a6 + a7));
+          tmem_wait_st();
+          tc_fence_before();
+          mbar_arrive(&bars.p_full[b]);
+          if (sparse) o_has[b] = true;
+        }
       }
     }
     if (ok) {
@@ -706,26 +1041,27 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       ok = __all_sync(0xffffffffu, ok);
     }
     if (!ok) record_timeout(p, &abort_flag);
-    float l_row[2];  // the row's whole sum: both halves, under the same max
+    float l_row[NT];  // the row's whole sum: both halves, under the same max
 #pragma unroll
-    for (int b = 0; b < 2; ++b) l_row[b] = l[b] + __shfl_xor_sync(0xffffffffu, l[b], 16);
+    for (int x = 0; x < NT; ++x)
+      l_row[x] = C::kOwnTile ? l[x] : l[x] + __shfl_xor_sync(0xffffffffu, l[x], 16);
     if (ns == 1) {
       if (ok) {
         tc_fence_after();
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          if (b == 1 && !has_q1) break;
+        for (int x = 0; x < NT; ++x) {
+          const int b = C::kOwnTile ? b_own : x;
+          if (b >= nb) break;
           const int token = (qt0 + b) * kTile + row;
           const bool in_range = token < p.T;
           __nv_bfloat16* orow = static_cast<__nv_bfloat16*>(p.out) +
                                 (((size_t)nd.q_index * p.T + token) * p.H + h) * D + DH * half;
-          const float inv_l = l_row[b] > 0.0f ? 1.0f / l_row[b] : 0.0f;  // no visible key: O = 0
+          const float inv_l = l_row[x] > 0.0f ? 1.0f / l_row[x] : 0.0f;  // no visible key: O = 0
 #pragma unroll
           for (int c = 0; c < DH / 32; ++c) {
             uint32_t o[32];
-            if (sparse ? o_has[b] : n_tiles > 0) {  // some key tile was attended
-              tmem_ld16x2_32<DH>(tbase + lane_off + col_o(b) + c * 32, o);
-              tmem_wait_ld(o);
+            if (sparse ? o_has[x] : n_tiles > 0) {  // some key tile was attended
+              ld_o(col_o<D>(b) + c * 32, o);
             } else {  // no key tile attended in this range (block-sparse): no MMA wrote O
 #pragma unroll
               for (int e = 0; e < 32; ++e) o[e] = 0u;
@@ -745,7 +1081,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           }
           if (p.lse != nullptr && in_range && half == 0)
             p.lse[((size_t)nd.q_index * p.H + h) * p.T + token] =
-                (m[b] + __log2f(l_row[b])) * 0.69314718055994531f;
+                (m[x] + __log2f(l_row[x])) * 0.69314718055994531f;
         }
       }
     } else {
@@ -757,16 +1093,16 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         tc_fence_after();
         float4* part4 = reinterpret_cast<float4*>(part);
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          if (b == 1 && !has_q1) break;
+        for (int x = 0; x < NT; ++x) {
+          const int b = C::kOwnTile ? b_own : x;
+          if (b >= nb) break;
           const int r = b * 128 + row;
-          const float inv_l = l_row[b] > 0.0f ? 1.0f / l_row[b] : 0.0f;  // no visible key here
+          const float inv_l = l_row[x] > 0.0f ? 1.0f / l_row[x] : 0.0f;  // no visible key here
 #pragma unroll
           for (int c = 0; c < DH / 32; ++c) {
             uint32_t o[32];
-            if (sparse ? o_has[b] : n_tiles > 0) {  // some key tile was attended
-              tmem_ld16x2_32<DH>(tbase + lane_off + col_o(b) + c * 32, o);
-              tmem_wait_ld(o);
+            if (sparse ? o_has[x] : n_tiles > 0) {  // some key tile was attended
+              ld_o(col_o<D>(b) + c * 32, o);
             } else {  // no key tile attended in this range (block-sparse): no MMA wrote O
 #pragma unroll
               for (int e = 0; e < 32; ++e) o[e] = 0u;
@@ -778,8 +1114,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
                               __uint_as_float(o[v * 4 + 2]) * inv_l, __uint_as_float(o[v * 4 + 3]) * inv_l);
           }
           if (half == 0) {
-            part[D * 256 + r] = m[b];
-            part[D * 256 + 256 + r] = l_row[b];
+            part[D * 256 + r] = m[x];
+            part[D * 256 + 256 + r] = l_row[x];
           }
         }
       }
@@ -797,8 +1133,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         __threadfence();
         const float* base = p.ws + (size_t)sunit * ns * kItem;
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          if (b == 1 && !has_q1) break;
+        for (int x = 0; x < NT; ++x) {
+          const int b = C::kOwnTile ? b_own : x;
+          if (b >= nb) break;
           const int r = b * 128 + row;
           const int token = (qt0 + b) * kTile + row;
           if (token >= p.T) continue;
@@ -827,7 +1164,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           // of, so every load of an iteration is in flight at once (a loop
           // that waited for each L2 round trip in turn took ~9 us per CTA).
 #pragma unroll 2
-          for (int c8 = half * (D / 16); c8 < (half + 1) * (D / 16); ++c8) {
+          for (int c8 = half * (DH / 8); c8 < (half + 1) * (DH / 8); ++c8) {
             float4 x[kMaxSplit], y[kMaxSplit];
 #pragma unroll
             for (int k = 0; k < kMaxSplit; ++k) {

@@ -299,6 +299,57 @@ __device__ __forceinline__ void mma_ts_warp(uint32_t d_tmem, uint32_t a_tmem, ui
       : "memory");
 }
 
+// Runs of MMAs over consecutive K slices with one election for the run (an
+// election per MMA costs the issuing warp about as long as a 128 x 64 x 16 MMA
+// takes the tensor pipe).  The first MMA accumulates where `accumulate` says,
+// the others always.
+//
+// Four smem x smem MMAs, descriptors `step` (in 16-byte units) apart; the first
+// overwrites D.
+__device__ __forceinline__ void mma_ss_warp_x4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                               uint64_t step, uint32_t idesc) {
+  asm volatile(
+      "{\n"
+      " .reg .pred z, t, e;\n"
+      " setp.ne.b32 z, 0, 0;\n"
+      " setp.eq.b32 t, 0, 0;\n"
+      " elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %5, %9, z;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %6, %9, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %3, %7, %9, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %4, %8, %9, t;\n"
+      "}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(a_desc + step), "l"(a_desc + 2 * step), "l"(a_desc + 3 * step),
+      "l"(b_desc), "l"(b_desc + step), "l"(b_desc + 2 * step), "l"(b_desc + 3 * step), "r"(idesc)
+      : "memory");
+}
+
+// Eight tmem x smem MMAs over 128 keys: A (packed bf16) advances by 8 columns,
+// B (MN-major, 128-byte rows) by 16 rows = 2048 bytes.
+__device__ __forceinline__ void mma_ts_warp_x8(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                               uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n"
+      " .reg .pred p, t, e;\n"
+      " setp.ne.b32 p, %18, 0;\n"
+      " setp.eq.b32 t, 0, 0;\n"
+      " elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %9, %17, p;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%2], %10, %17, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%3], %11, %17, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%4], %12, %17, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%5], %13, %17, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%6], %14, %17, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%7], %15, %17, t;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%8], %16, %17, t;\n"
+      "}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "r"(a_tmem + 8), "r"(a_tmem + 16), "r"(a_tmem + 24), "r"(a_tmem + 32),
+      "r"(a_tmem + 40), "r"(a_tmem + 48), "r"(a_tmem + 56), "l"(b_desc), "l"(b_desc + 128),
+      "l"(b_desc + 256), "l"(b_desc + 384), "l"(b_desc + 512), "l"(b_desc + 640),
+      "l"(b_desc + 768), "l"(b_desc + 896), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 __device__ __forceinline__ void mma_commit_warp(uint64_t* bar) {
   asm volatile(
       "{\n"
