@@ -229,6 +229,57 @@ struct TileWalk {
   }
 };
 
+// The lowest n bits (none for n <= 0, all 32 for n >= 32).
+__device__ __forceinline__ uint32_t first_bits(int n) {
+  return n >= 32 ? ~0u : (n <= 0 ? 0u : (1u << n) - 1u);
+}
+
+// -inf where a key's bit is clear: bit e of w[c] belongs to s[c][e].
+template <int NC>
+__device__ __forceinline__ void hide_keys(uint32_t (&s)[NC][32], const uint32_t (&w)[NC]) {
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      if (!((w[c] >> e) & 1u)) s[c][e] = 0xFF800000u;
+}
+
+template <int NC>
+__device__ __forceinline__ float max_score(const uint32_t (&s)[NC][32]) {
+  float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+#pragma unroll
+    for (int e = 0; e < 32; e += 8) {
+      const int k = (c & 1) * 2 + (e >> 4);
+      mx[k] = max3(mx[k], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
+      mx[k] = max3(mx[k], __uint_as_float(s[c][e + 2]), __uint_as_float(s[c][e + 3]));
+      mx[k] = max3(mx[k], __uint_as_float(s[c][e + 4]), __uint_as_float(s[c][e + 5]));
+      mx[k] = max3(mx[k], __uint_as_float(s[c][e + 6]), __uint_as_float(s[c][e + 7]));
+    }
+  return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+}
+
+// Masks of one tile, for a whole warp.  w: this thread's visible keys; m_part:
+// the maximum of its unmasked scores, replaced by the maximum that the running
+// max m (log2 units, sl2 per unit of score) has to be compared with.  A warp
+// whose rows all see every key of the tile is left alone.  Otherwise the
+// hidden scores become -inf, and the maximum over the rest is only taken when
+// some row's unmasked maximum exceeds its m by the rescale threshold: below
+// that m does not move whatever the mask hides, so any smaller value (-inf)
+// has the same effect.  (Selecting and taking the maximum for every tile that
+// could hold a masked key took 2.2 times a dense tile.)
+template <int NC>
+__device__ __forceinline__ void mask_tile(uint32_t (&s)[NC][32], const uint32_t (&w)[NC],
+                                          float& m_part, float m, float sl2) {
+  uint32_t all = w[0];
+#pragma unroll
+  for (int c = 1; c < NC; ++c) all &= w[c];
+  if (!__any_sync(0xffffffffu, all != ~0u)) return;
+  hide_keys(s, w);
+  m_part = __any_sync(0xffffffffu, m_part * sl2 > m + kRescaleThreshold) ? max_score(s) : -INFINITY;
+}
+
 __device__ __forceinline__ void record_timeout(const AttnParams& p, volatile int* abort_flag) {
   *abort_flag = 1;
   atomicCAS(p.status, kStatusOk, kStatusTimeout);
@@ -692,18 +743,43 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     TileWalk<kSparse ? kMaskWords : 1> walk;
     if constexpr (sparse) walk.start(tmask, t_begin, n_all);
     int kt = sparse ? walk.next() : t_begin;  // key tile of the node
+    // Key state (0 own, then the visible contexts) of a key tile: a division
+    // by a reciprocal, exact for the tiles of the masked instances (kt < 2^12,
+    // nt_slot <= 2^9).
+    const uint32_t inv_nt = p.nt_slot > 1 ? 0xFFFFFFFFu / (uint32_t)p.nt_slot + 1u : 0u;
+    auto state_of = [&](int tile) { return inv_nt ? (int)__umulhi((uint32_t)tile, inv_nt) : tile; };
+    // Token-mask instance: this thread's bits of its row for a key tile, from
+    // the own-chunk mask or from the history mask of the tile's key state (the
+    // caller's context index); all ones without such a mask.  Each is fetched
+    // a key tile ahead of its use: its L2 latency, on the path from S to P,
+    // cost about 0.1 us a tile.
+    auto token_bits = [&](int b, int tile, uint32_t (&ow)[NC]) {
+#pragma unroll
+      for (int c = 0; c < NC; ++c) ow[c] = ~0u;
+      const int st = state_of(tile);
+      const uint32_t* mask = st == 0 ? p.own_mask : p.hist_mask;
+      const int u = (qt0 + b) * kTile + row;
+      if (mask != nullptr && u < p.T) {  // rows past T are never stored
+        const size_t qrow = (size_t)nd.q_index * p.T + u;
+        const uint32_t* mrow =
+            mask + (st == 0 ? qrow * p.own_words
+                            : (qrow * p.hist_states + (nd.src[st] - 1)) * p.hist_words);
+        const int words = st == 0 ? p.own_words : p.hist_words;
+        const int wi = (tile - st * p.nt_slot) * 4 + half * 2;  // first key of this thread / 32
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ow[c] = wi + c < words ? __ldg(mrow + wi + c) : 0u;
+      }
+    };
     if constexpr (C::kOwnTile) {
       const int b = b_own;
       int kst = kt / p.nt_slot;                 // its key state: 0 own, then the visible contexts
       int t = kt - kst * p.nt_slot;             // and its place in the state's slot
       // Steps to the next key tile of the walk.  A dense walk visits the tiles
       // of a slot in order (with the frame-causal gap at the end of the own
-      // slot), so no division is needed; a block-sparse one divides by a
-      // reciprocal (exact: kt < 2^12 and nt_slot <= 2^9).
-      const uint32_t inv_nt = p.nt_slot > 1 ? 0xFFFFFFFFu / (uint32_t)p.nt_slot + 1u : 0u;
+      // slot), so no division is needed.
       auto advance = [&](int next) {
         if constexpr (sparse) {
-          kst = inv_nt ? (int)__umulhi((uint32_t)next, inv_nt) : next;
+          kst = state_of(next);
           t = next - kst * p.nt_slot;
         } else {
           t += next - kt;
@@ -720,66 +796,28 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       auto wait_s = [&](int bar, uint32_t par) {
         return __all_sync(0xffffffffu, mbar_wait(&bars.s_full[b * 3 + bar], par, &abort_flag, tmo)) != 0;
       };
-      // token-level mask (token-mask instance): this thread's bits of its row
-      // for the key tile, from the own-chunk mask or from the history mask of
-      // the tile's key state (the caller's context index)
-      auto token_bits = [&](uint32_t (&ow)[NC]) {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) ow[c] = ~0u;
-        if constexpr (kOwn) {
-          const bool masked = (kst == 0 ? p.own_mask : p.hist_mask) != nullptr;
-          const int u = (qt0 + b) * kTile + row;
-          if (masked && u < p.T) {  // rows past T are never stored
-            const size_t qrow = (size_t)nd.q_index * p.T + u;
-            const uint32_t* mrow =
-                kst == 0 ? p.own_mask + qrow * p.own_words
-                         : p.hist_mask + (qrow * p.hist_states + (nd.src[kst] - 1)) * p.hist_words;
-            const int words = kst == 0 ? p.own_words : p.hist_words;
-            const int wi = t * 4;  // key 128 t of the state
-#pragma unroll
-            for (int c = 0; c < NC; ++c) ow[c] = wi + c < words ? __ldg(mrow + wi + c) : 0u;
-          }
-          return masked;
-        }
-        return false;
-      };
       // One step from its scores s (with the maximum cmax of each 32-key chunk)
       // up to the row's running max: masks, then moves m and rescales O and l
       // where a row needs it.  False: a wait expired.
       auto row_max = [&](int i, uint32_t (&s)[NC][32], const float (&cmax)[NC],
-                         const uint32_t (&ow)[NC], bool own_tile) {
+                         const uint32_t (&ow)[NC]) {
         float m_part = cmax[0];
 #pragma unroll
         for (int c = 1; c < NC; ++c) m_part = fmaxf(m_part, cmax[c]);
         const int valid_tile = (t == p.nt_slot - 1) ? p.valid_last : kTile;
         const bool own_fc = frame_causal && kst == 0;
         // The loads also reduce each 32-column chunk to its maximum, so a full
-        // tile needs no max tree; tiles that can hold masked keys (a slot's
-        // ragged last tile, the own chunk under frame causality) take the max
-        // over what is left after masking.  The test is the same for every
-        // thread, so it needs no vote.
-        if (valid_tile < kTile || own_fc || own_tile) {
+        // tile needs no max tree.  Tiles that can hold masked keys (a slot's
+        // ragged last tile, the own chunk under frame causality, token masks)
+        // take mask_tile; the test is the same for every thread.
+        if (kOwn || valid_tile < kTile || own_fc) {
           // own-chunk tile under frame causality: keys up to the end of this
           // row's latent frame are visible (tile 0, frame 0, always is)
           const int valid = own_fc ? min(valid_tile, frame_end[0] - t * kTile) : valid_tile;
-          const int vrel = valid;
-          float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+          uint32_t w[NC];
 #pragma unroll
-          for (int c = 0; c < NC; ++c)
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (c * 32 + e >= vrel || !((ow[c] >> e) & 1u)) s[c][e] = __float_as_uint(-INFINITY);
-#pragma unroll
-          for (int c = 0; c < NC; ++c)
-#pragma unroll
-            for (int e = 0; e < 32; e += 8) {
-              const int k = (c & 1) * 2 + (e >> 4);
-              mx[k] = max3(mx[k], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
-              mx[k] = max3(mx[k], __uint_as_float(s[c][e + 2]), __uint_as_float(s[c][e + 3]));
-              mx[k] = max3(mx[k], __uint_as_float(s[c][e + 4]), __uint_as_float(s[c][e + 5]));
-              mx[k] = max3(mx[k], __uint_as_float(s[c][e + 6]), __uint_as_float(s[c][e + 7]));
-            }
-          m_part = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          for (int c = 0; c < NC; ++c) w[c] = ow[c] & first_bits(valid - c * 32);
+          mask_tile(s, w, m_part, m[0], sl2);
         }
         const float m_tile = m_part * sl2;
         const float m_new = fmaxf(m[0], m_tile);
@@ -844,6 +882,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       const int my_tiles = b < nb ? n_tiles : 0;
       int buf = b, bar = 0;  // S buffer of step n = nb * i + b; i % 3 and that barrier's phase
       uint32_t par = 0;
+      uint32_t ow[NC];  // token masks: the bits of key tile kt
+#pragma unroll
+      for (int c = 0; c < NC; ++c) ow[c] = ~0u;
+      if constexpr (kOwn)
+        if (my_tiles > 0) token_bits(b, kt, ow);
       for (int i = 0; ok && i < my_tiles; ++i) {
         const int kt_next = sparse ? walk.next() : next_kt(kt);
         uint64_t* p_bar = &bars.p_full[b * 3 + bar];
@@ -860,10 +903,10 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 #pragma unroll
           for (int c = 0; c < NC; ++c) tmem_wait_ld(s[c]);
           tmem_wait_ld_max(cmax);
-          uint32_t ow[NC];
-          const bool own_tile = token_bits(ow);
-          ok = row_max(i, s, cmax, ow, own_tile);
+          ok = row_max(i, s, cmax, ow);
           if (!ok) break;
+          if constexpr (kOwn)
+            if (i + 1 < my_tiles) token_bits(b, kt_next, ow);
           const uint64_t negm = neg_max();
           uint64_t acc[4] = {0, 0, 0, 0};
           expo(s[0], negm, acc);
@@ -876,6 +919,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           tc_fence_before();
           add_sum(acc);
           o_has[0] = true;
+        } else if constexpr (kOwn) {
+          if (i + 1 < my_tiles) token_bits(b, kt_next, ow);
         }
         mbar_arrive(p_bar);
         advance(kt_next);
@@ -888,6 +933,14 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       }
     } else {
       int kt_next = kt;
+      uint32_t ow[2][NC];  // token masks: the bits of key tile kt per query tile
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ow[b][c] = ~0u;
+        if constexpr (kOwn)
+          if (n_tiles > 0) token_bits(b, kt, ow[b]);
+      }
       for (int i = 0; ok && i < n_tiles; ++i, kt = kt_next) {
         // The next tile of the walk and, under a tile mask, which query tiles
         // attend this one: read from shared memory before the S wait, so their
@@ -899,29 +952,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         const int t = kt % p.nt_slot;  // key tile inside its slot
         const int valid_tile = (t == p.nt_slot - 1) ? p.valid_last : kTile;
         const bool own_fc = frame_causal && kt < p.nt_slot;
-  #pragma unroll
+#pragma unroll
         for (int b = 0; b < 2; ++b) {
           if (b == 1 && !has_q1) break;
-          // token-level mask (token-mask instance): this thread's 64 bits of its
-          // row for this key tile, from the own-chunk mask or from the history
-          // mask of the tile's key state (the caller's context index); fetched
-          // before the wait so that the load hides behind it
-          const int kst = kOwn ? kt / p.nt_slot : 0;  // key state: 0 own, then the visible contexts
-          const bool own_tile = kOwn && (kst == 0 ? p.own_mask : p.hist_mask) != nullptr;
-          uint32_t ow[2] = {~0u, ~0u};
-          if (own_tile) {
-            const int u = (qt0 + b) * kTile + row;
-            if (u < p.T) {  // rows past T are never stored
-              const size_t qrow = (size_t)nd.q_index * p.T + u;
-              const uint32_t* mrow =
-                  kst == 0 ? p.own_mask + qrow * p.own_words
-                           : p.hist_mask + (qrow * p.hist_states + (nd.src[kst] - 1)) * p.hist_words;
-              const int words = kst == 0 ? p.own_words : p.hist_words;
-              const int wi = (kt - kst * p.nt_slot) * 4 + half * 2;  // key 128 t + 64 half of the state
-              ow[0] = wi < words ? __ldg(mrow + wi) : 0u;
-              ow[1] = wi + 1 < words ? __ldg(mrow + wi + 1) : 0u;
-            }
-          }
           ok = mbar_wait(&bars.s_full[b], (uint32_t)i & 1u, &abort_flag, tmo);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
@@ -932,19 +965,15 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           if (sparse && !((attends >> b) & 1u)) {
             // query tile b skips this key tile: no S was computed, no P is due
             mbar_arrive(&bars.p_full[b]);
+            if constexpr (kOwn)
+              if (i + 1 < n_tiles) token_bits(b, kt_next, ow[b]);
             continue;
           }
           tc_fence_after();
           const uint32_t scol = tbase + lane_off + col_s<D>(b);
           const uint32_t ocol = tbase + lane_off + col_o<D>(b);
-          // own-chunk tile under frame causality: keys up to the end of this
-          // row's latent frame are visible (tile 0, frame 0, always is)
-          const int valid = own_fc ? min(valid_tile, frame_end[b] - t * kTile) : valid_tile;
-          const int vrel = valid - half * 64;  // visible keys among this thread's 64
           // The loads also reduce each 32-column chunk to its maximum, so a
-          // full tile needs no max tree; a tile with masked keys (the ragged
-          // last tile of a slot, frame causality) takes the max over what is
-          // left after masking.
+          // full tile needs no max tree.
           uint32_t s[2][32];
           float cmax[2];
           tmem_ld16x2_32_max<64>(scol, s[0], cmax[0]);
@@ -954,26 +983,17 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           tmem_wait_ld_max2(cmax);
           float m_part = fmaxf(cmax[0], cmax[1]);
           // Tiles that can hold masked keys (a slot's ragged last tile, the own
-          // chunk under frame causality) take the masked path; the test is the
-          // same for every thread, so it needs no vote.
-          if (valid_tile < kTile || own_fc || own_tile) {
-            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-  #pragma unroll
-            for (int c = 0; c < 2; ++c)
-  #pragma unroll
-              for (int e = 0; e < 32; ++e)
-                if (c * 32 + e >= vrel || !((ow[c] >> e) & 1u)) s[c][e] = __float_as_uint(-INFINITY);
-  #pragma unroll
-            for (int c = 0; c < 2; ++c)
-  #pragma unroll
-              for (int e = 0; e < 32; e += 8) {
-                const int k = (c & 1) * 2 + (e >> 4);
-                mx[k] = max3(mx[k], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
-                mx[k] = max3(mx[k], __uint_as_float(s[c][e + 2]), __uint_as_float(s[c][e + 3]));
-                mx[k] = max3(mx[k], __uint_as_float(s[c][e + 4]), __uint_as_float(s[c][e + 5]));
-                mx[k] = max3(mx[k], __uint_as_float(s[c][e + 6]), __uint_as_float(s[c][e + 7]));
-              }
-            m_part = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+          // chunk under frame causality, token masks) take mask_tile; the test
+          // is the same for every thread.
+          if (kOwn || valid_tile < kTile || own_fc) {
+            // own-chunk tile under frame causality: keys up to the end of this
+            // row's latent frame are visible (tile 0, frame 0, always is)
+            const int valid = own_fc ? min(valid_tile, frame_end[b] - t * kTile) : valid_tile;
+            const int vrel = valid - half * 64;  // visible keys among this thread's 64
+            const uint32_t w[2] = {ow[b][0] & first_bits(vrel), ow[b][1] & first_bits(vrel - 32)};
+            mask_tile(s, w, m_part, m[b], sl2);
+            if constexpr (kOwn)
+              if (i + 1 < n_tiles) token_bits(b, kt_next, ow[b]);
           }
           const float m_tile = fmaxf(m_part, __shfl_xor_sync(0xffffffffu, m_part, 16)) * sl2;
           const float m_new = fmaxf(m[b], m_tile);
@@ -986,12 +1006,12 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
             if (sparse ? o_has[b] : i > 0) {
               // O_b holds the sum over earlier tiles: the commit that completed
               // S_b of this tile came after PV_b of the previous one.
-  #pragma unroll
+#pragma unroll
               for (int c = 0; c < DH / 32; ++c) {
                 uint32_t o[32];
                 tmem_ld16x2_32<DH>(ocol + c * 32, o);
                 tmem_wait_ld(o);
-  #pragma unroll
+#pragma unroll
                 for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
                 tmem_st16x2_32<DH>(ocol + c * 32, o);
               }
@@ -1010,9 +1030,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           // the same registers (word e/2 is written after elements e, e+1 are
           // read); the two halves make one 32-column store over S (keys
           // 0..63 of the row at columns 0..31, keys 64..127 at 32..63).
-  #pragma unroll
+#pragma unroll
           for (int c = 0; c < 2; ++c) {
-  #pragma unroll
+#pragma unroll
             for (int e = 0; e < 32; e += 2) {
               float x0, x1;
               ffma2(x0, x1, __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]), sl2x2, negm);
