@@ -370,11 +370,14 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     // Gather the caller's mask rows of the two query tiles into the kernel's
     // key tile order (slot list without hidden context slots), then take
     // this split's share of the union's set bits.  Without a tile mask every
-    // key tile is kept.
+    // key tile is kept that the token masks leave something of.
     const int words = (n_all + 31) >> 5;  // <= kMaskWords, checked on the host
     const uint32_t* row0 =
         p.tile_mask ? p.tile_mask + ((size_t)nd.q_index * p.n_qt + qt0) * p.mask_words : nullptr;
     const uint32_t* row1 = row0 ? row0 + p.mask_words : nullptr;
+    const uint8_t* any0 =
+        p.any_tile ? p.any_tile + ((size_t)nd.q_index * p.n_qt + qt0) * p.any_stride : nullptr;
+    const uint8_t* any1 = any0 ? any0 + p.any_stride : nullptr;
     int total = 0;
     for (int w = 0; w < words; ++w) {
       const int i = (w << 5) + lane;
@@ -384,6 +387,10 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         const int k = nd.src[s] * p.nt_slot + (i - s * p.nt_slot);
         b0 = row0 ? ((row0[k >> 5] >> (k & 31)) & 1u) != 0u : true;
         if (has_q1) b1 = row1 ? ((row1[k >> 5] >> (k & 31)) & 1u) != 0u : true;
+        if (any0) {
+          b0 = b0 && any0[k] != 0;
+          b1 = b1 && any1[k] != 0;
+        }
       }
       const uint32_t m0 = __ballot_sync(0xffffffffu, b0);
       const uint32_t m1 = __ballot_sync(0xffffffffu, b1);

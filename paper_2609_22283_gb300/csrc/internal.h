@@ -65,8 +65,23 @@ struct alignas(128) AttnParams {
   const uint32_t* hist_mask;
   int32_t hist_states;
   int32_t hist_words;
+  // Key tiles that the token masks leave anything of, a byte per (node, query
+  // tile, key tile in the order of tile_mask), rows of any_stride bytes, or null
+  const uint8_t* any_tile;
+  int32_t any_stride;
   int32_t masked;             // a tile or token mask given: a masked kernel instance
   AttnNode nodes[SVA_MAX_NODES];
+};
+
+// Reduction of the token masks to the bytes of AttnParams::any_tile.
+struct ScanParams {
+  const uint32_t* own_mask;   // as in AttnParams
+  const uint32_t* hist_mask;
+  int32_t own_words, hist_states, hist_words;
+  int32_t T, n_qt;
+  uint8_t* any;
+  int32_t row_bytes;
+  int32_t n_ctx[SVA_MAX_NODES];  // context states per node, hidden ones included
 };
 
 struct RopeNode {
@@ -102,6 +117,8 @@ cudaError_t static_split_scratch(int device, void** ptr);
 
 // Launchers (defined in the .cu files).  They return the launch error.
 cudaError_t launch_attend(const AttnParams& p, int head_dim, int grid, cudaStream_t s);
+// `max_states`: 1 + the largest n_ctx.
+cudaError_t launch_mask_scan(const ScanParams& p, int n_nodes, int max_states, cudaStream_t s);
 cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s);
 
 }  // namespace sva

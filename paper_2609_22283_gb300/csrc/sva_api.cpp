@@ -267,6 +267,12 @@ size_t ws_total_bytes(const sva_cache* c) {
   return ws_counter_bytes(c) + (size_t)ws_items(c) * ws_item_bytes(c);
 }
 
+// Workspace items that the scan of token masks may take from the split
+// partials.  A plan splits at most one wave of units 4 ways, so it leaves 4 of
+// the 4 waves of items over.
+constexpr long long kScanItems = 4;
+constexpr long long kScanMinTiles = 12000;
+
 // Fewest key tiles a work unit of node i walks: all of its slots' tiles,
 // except under frame causality, where a pair of query tiles skips the own
 // chunk's tiles past its last row's frame (the first pair skips the most).
@@ -749,7 +755,23 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
     min_tiles = std::min(min_tiles, key_tiles_walked(c, p.nodes[i], p.nt_slot));
   p.n_qp = (p.n_qt + 1) / 2;
   const long long units = (long long)g.num_heads * n_nodes * p.n_qp;
-  const long long cap = (scratch == Scratch::kStatic || c->ws != nullptr) ? ws_items(c) : 0;
+  long long cap = (scratch == Scratch::kStatic || c->ws != nullptr) ? ws_items(c) : 0;
+  // A launch with token masks scans them first for the key tiles they leave
+  // anything of, when a workspace can take the result and the launch is long
+  // enough for the scan's 3-5 us to be lost in it: kScanMinTiles walks of a
+  // key tile by a query-tile pair, about 100 us of attention.
+  int max_states = 1;
+  for (int i = 0; i < n_nodes; ++i) max_states = std::max(max_states, 1 + nodes[i].n_ctx);
+  size_t scan_bytes = 0;
+  if ((p.own_mask != nullptr || p.hist_mask != nullptr) && c->ws != nullptr &&
+      scratch == Scratch::kWorkspace && units * min_tiles >= kScanMinTiles) {
+    const size_t bytes = round_up((size_t)n_nodes * p.n_qt * max_states * p.nt_slot, 256);
+    const long long items = (long long)((bytes + ws_item_bytes(c) - 1) / ws_item_bytes(c));
+    if (items <= kScanItems) {
+      scan_bytes = bytes;
+      cap -= items;
+    }
+  }
   long long n_full = 0;
   int n_split = 1;
   plan_split(c, units, min_tiles, cap, &n_full, &n_split);
@@ -809,6 +831,25 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
       cudaError_t e = cudaMemsetAsync(split_base, 0, counter_bytes, reinterpret_cast<cudaStream_t>(s));
       if (e != cudaSuccess) return cuda_fail(e, "clearing the split counters");
     }
+  }
+  // Token masks: reduce them to the key tiles they leave anything of, in the
+  // last scan_bytes of the workspace (the split items end before, see `cap`).
+  if (scan_bytes > 0) {
+    static thread_local sva::ScanParams sp;
+    sp.own_mask = p.own_mask;
+    sp.hist_mask = p.hist_mask;
+    sp.own_words = p.own_words;
+    sp.hist_states = p.hist_states;
+    sp.hist_words = p.hist_words;
+    sp.T = c->L.T;
+    sp.n_qt = p.n_qt;
+    sp.any = reinterpret_cast<uint8_t*>(c->ws) + ws_total_bytes(c) - scan_bytes;
+    sp.row_bytes = max_states * p.nt_slot;
+    for (int i = 0; i < n_nodes; ++i) sp.n_ctx[i] = nodes[i].n_ctx;
+    p.any_tile = sp.any;
+    p.any_stride = sp.row_bytes;
+    cudaError_t e = sva::launch_mask_scan(sp, n_nodes, max_states, reinterpret_cast<cudaStream_t>(s));
+    if (e != cudaSuccess) return cuda_fail(e, "mask scan launch");
   }
   const long long grid = n_full + (units - n_full) * n_split;
   cudaError_t e = sva::launch_attend(p, g.head_dim, (int)grid, reinterpret_cast<cudaStream_t>(s));

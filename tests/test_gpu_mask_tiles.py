@@ -75,3 +75,84 @@ def test_hidden_large_keys(T, W, pattern, d, split):
     assert (lse[0][none] == -math.inf).all()
     assert ((lse[0].double() - ref)[~none].abs() <= 2e-3 + 2.0 ** -20 * ref[~none].abs()).all()
     cache.close()
+
+
+# Launches long enough for the masks to be scanned for empty key tiles first (with a workspace)
+# against the same call without a workspace, which walks every tile: T = 2500 (20 tiles, the last of
+# 68 rows; 78.1 mask words), 12 heads, one or two nodes.  Both paths multiply the same tiles that
+# hold a visible key, so they differ by the key-range split alone: two bf16 roundings of O and the
+# rounding of P relative to another maximum.
+SCAN_FORMS = {
+    "both": {},
+    "own only": {"hist": False},
+    "history only": {"own": False},
+    "hidden context": {"visible": [1, 0, 1, 1]},
+    "long rows": {"extra": 3, "states": 6},
+    "tile mask too": {"tiles": True},
+    "frame causal": {"causal": True},
+    "two nodes": {"n": 2},
+}
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("form", sorted(SCAN_FORMS))
+def test_scan_of_empty_tiles(form, d):
+    f = SCAN_FORMS[form]
+    F, Hp, Wp, H, W, n = 4, 25, 25, 12, 4, f.get("n", 1)
+    T, nt = F * Hp * Wp, 20
+    assert H * n * 10 * (W + 1) * nt >= 12000    # the size from which masks are scanned
+    g = sva.make_geometry(H, d, F, Hp, Wp, num_slots=W + n, pairs=rope_pairs_for(d), max_frames=F * (W + 3))
+    cache = sva.Cache(g)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    draw = lambda: torch.randn((1, T, H, d), generator=gen, device="cuda").bfloat16()  # noqa: E731
+    ctx, entries = [], []
+    for j in range(W):
+        s = cache.bind(0, W - j, 0)
+        cache.rope_kv_write([dict(seq=0, chunk=W - j, level=0, own_slot=s)], draw(), draw())
+        ctx.append(s)
+    for i in range(n):
+        s = cache.bind(0, W + 1, i)
+        cache.rope_kv_write([dict(seq=0, chunk=W + 1, level=i, own_slot=s)], draw(), draw())
+        entries.append(dict(seq=0, chunk=W + 1, level=i, own_slot=s, ctx=ctx[:W - i],
+                            visible=f.get("visible", [1] * W)[:W - i], within=int(f.get("causal", False))))
+    nodes = sva.make_nodes(entries)
+    q = torch.cat([draw() for _ in range(n)])
+
+    # blocks of 100 queries x 200 keys, one in four kept, one state wholly hidden, junk past T
+    def words(states, extra):
+        m = torch.rand((n, T // 100, states, T // 200 + 1), generator=gen, device="cuda") < 0.25
+        m = m.repeat_interleave(100, 1).repeat_interleave(200, 3)[..., :T]
+        m[:, :, states - 1] = False
+        m[:, 300:420] = False                       # a run of queries across a tile edge that see nothing
+        full = torch.ones(m.shape[:-1] + (-(-T // 32) * 32 + 32 * extra,), dtype=torch.bool, device="cuda")
+        full[..., :T] = m
+        return pack_bits(full.cpu(), full.shape[-1] // 32).cuda()
+
+    extra, states = f.get("extra", 0), f.get("states", W)
+    own = words(2, extra)[:, :, 0].contiguous() if f.get("own", True) else None
+    hist = words(states, extra) if f.get("hist", True) else None
+    tile = None
+    if f.get("tiles"):
+        keep = torch.rand((n, nt, (1 + W) * nt), generator=gen, device="cuda") < 0.7
+        tile = pack_bits(keep.cpu(), -(-(1 + W) * nt // 32)).cuda()
+    got = []
+    for ws in (False, True):
+        if ws:
+            buf = torch.full((cache.workspace_bytes(),), 255, dtype=torch.uint8, device="cuda")
+            cache.set_workspace(buf)
+        for _ in range(2):     # the second call finds the first one's bytes in the workspace
+            out = torch.full_like(q, float("nan"))
+            lse = torch.full((n, H, T), float("nan"), device="cuda")
+            cache.attend_nodes_masked(nodes, q, out, lse, tile_mask=tile, own_mask=own, hist_mask=hist)
+        assert cache.poll() == sva.OK
+        got.append((out.double(), lse.double()))
+    (a, la), (b, lb) = got
+    none = la == -math.inf
+    assert torch.equal(none, lb == -math.inf)
+    assert ((la - lb)[~none].abs() <= 1e-3).all()
+    assert not a.isnan().any() and not b.isnan().any()
+    # the results' roundings, and P's in either path: at most 2^-9 E_p|V| <= 2^-9 max |V|
+    v_max = float(cache.slot_pool()[:, 1].abs().max())
+    assert ((a - b).abs() <= 2.0 ** -9 * (a.abs() + b.abs()) + 2 * 2.0 ** -9 * v_max).all()
+    assert float((a - b).norm() / b.norm()) <= 5e-3
+    cache.close()
