@@ -328,8 +328,9 @@ sva_status sva_attend_nodes_masked(sva_cache* c, const sva_node* nodes, int32_t 
 
 /* Bytes of the optional split workspace of a cache (0 if c is NULL).  With
  * a workspace attached, sva_attend_nodes may divide each (node, head,
- * query-tile pair) work unit into up to 4 contiguous key ranges computed by
- * separate CTAs and merged on the device (the softmax of Eq. 4 recombined
+ * query-tile pair) work unit into contiguous key ranges (up to 4, or up to 8
+ * where all fit on the GPU at once) computed by separate CTAs and merged on
+ * the device (the softmax of Eq. 4 recombined
  * from per-range maxima and sums), which fills the GPU when a launch has
  * too few work units; results agree with the unsplit computation to
  * rounding. */

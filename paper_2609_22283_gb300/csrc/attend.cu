@@ -287,9 +287,11 @@ __device__ __forceinline__ void record_timeout(const AttnParams& p, volatile int
 
 // Instances: kSparse = a block-sparse tile mask is walked (all ones when the
 // caller gives none); kOwn = a token-level mask inside the own chunk is
-// applied (only with kSparse).  Each extra feature costs the per-tile loop,
-// so a launch takes the leanest instance that covers it.
-template <int D, bool kSparse, bool kOwn>
+// applied (only with kSparse); kCluster = every unit is split over the CTAs of
+// one cluster, which merge through their shared memory.  Each extra feature
+// costs the per-tile loop, so a launch takes the leanest instance that covers
+// it.
+template <int D, bool kSparse, bool kOwn, bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_constant__ AttnParams p) {
   using C = AttnCfg<D>;
   extern __shared__ uint8_t smem_raw[];
@@ -306,7 +308,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   // Work unit, head-major so the CTAs that share a head's K/V run together.
   // The first n_full units run unsplit (one CTA each, the full waves); the
   // others are split n_split ways, the splits of a unit adjacent.
-  const bool whole = (int)blockIdx.x < p.n_full;
+  // kCluster: one cluster of n_split CTAs per unit (n_full = 0).
+  const bool whole = !kCluster && (int)blockIdx.x < p.n_full;
   const int ns = whole ? 1 : p.n_split;  // key ranges of this unit
   const int split = whole ? 0 : (int)(blockIdx.x - p.n_full) % p.n_split;
   const int unit = whole ? (int)blockIdx.x : p.n_full + (int)(blockIdx.x - p.n_full) / p.n_split;
@@ -658,6 +661,10 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     }
     // ---------------------------------------------------------------- teardown (warpgroup 0)
     __syncwarp();
+    if constexpr (kCluster) {  // the two barriers of the merge
+      cluster_sync();
+      cluster_sync();
+    }
     tc_fence_before();
     __syncthreads();
     if (abort_flag) {
@@ -1072,7 +1079,103 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 #pragma unroll
     for (int x = 0; x < NT; ++x)
       l_row[x] = C::kOwnTile ? l[x] : l[x] + __shfl_xor_sync(0xffffffffu, l[x], 16);
-    if (ns == 1) {
+    if constexpr (kCluster) {
+      // Merge over distributed shared memory.  Every CTA owns 1/ns of the
+      // output columns (whole groups of 8) for all 256 rows; each pushes its
+      // normalised fp32 partial, and every row's m and l, to the owners, into
+      // the shared memory that Q, K and V no longer need, and each owner adds
+      // up its columns in order of the key ranges.  So the merge is spread
+      // over the unit's CTAs (131 KB out and in per CTA at D = 128, whatever
+      // ns), needs no workspace, and costs two cluster barriers instead of
+      // stores to L2, a fence, an atomic and the last CTA's reads.
+      constexpr int kGroups8 = D / 8;
+      const int per = (kGroups8 + ns - 1) / ns;  // column groups per owner
+      const uint32_t data = smem_u32(smem);
+      const uint32_t ml = data + (uint32_t)(ns * per) * 8192u;  // [ns][m, l][256] fp32
+      __syncwarp();
+      cluster_sync();  // every CTA's MMAs are complete: its tiles may be overwritten
+      if (ok) {
+        tc_fence_after();
+#pragma unroll
+        for (int x = 0; x < NT; ++x) {
+          const int b = C::kOwnTile ? b_own : x;
+          if (b >= nb) break;
+          const int r = b * 128 + row;
+          const float inv_l = l_row[x] > 0.0f ? 1.0f / l_row[x] : 0.0f;  // no visible key here
+#pragma unroll
+          for (int c = 0; c < DH / 32; ++c) {
+            uint32_t o[32];
+            if (sparse ? o_has[x] : n_tiles > 0) {  // some key tile was attended
+              ld_o(col_o<D>(b) + c * 32, o);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 32; ++e) o[e] = 0u;
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+              const int g8 = (DH * half + c * 32) / 8 + v;
+              const int owner = g8 / per;
+              const uint32_t dst = mapa_shared(
+                  data + (uint32_t)((split * per + g8 - owner * per) * 8192 + r * 16), (uint32_t)owner);
+#pragma unroll
+              for (int q = 0; q < 2; ++q)
+                st_cluster_v4(dst + q * 4096, __uint_as_float(o[v * 8 + q * 4]) * inv_l,
+                              __uint_as_float(o[v * 8 + q * 4 + 1]) * inv_l,
+                              __uint_as_float(o[v * 8 + q * 4 + 2]) * inv_l,
+                              __uint_as_float(o[v * 8 + q * 4 + 3]) * inv_l);
+            }
+          }
+          if (half == 0)
+            for (int k = 0; k < ns; ++k) {
+              const uint32_t dst = mapa_shared(ml + (uint32_t)(split * 2048 + r * 4), (uint32_t)k);
+              st_cluster_f32(dst, m[x]);
+              st_cluster_f32(dst + 1024, l_row[x]);
+            }
+        }
+      }
+      __syncwarp();
+      cluster_sync();  // every partial has arrived; nothing is read from another CTA after this
+      const int r = threadIdx.x - 128;  // this thread's row of the pair
+      const int token = qt0 * kTile + r;
+      if (ok && token < p.T && r < nb * kTile) {
+        float M = -INFINITY;
+        for (int k = 0; k < ns; ++k) M = fmaxf(M, ld_shared_f32(ml + (uint32_t)(k * 2048 + r * 4)));
+        const float M_sub = (M == -INFINITY) ? 0.0f : M;  // every range empty: O = 0
+        float w[kMaxClusterSplit];
+        float L = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kMaxClusterSplit; ++k) {
+          w[k] = 0.0f;
+          if (k < ns) {
+            const uint32_t at = ml + (uint32_t)(k * 2048 + r * 4);
+            w[k] = ld_shared_f32(at + 1024) * ex2(ld_shared_f32(at) - M_sub);
+            L += w[k];
+          }
+        }
+        const float inv_L = L > 0.0f ? 1.0f / L : 0.0f;
+        uint4* orow4 = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) +
+                                                (((size_t)nd.q_index * p.T + token) * p.H + h) * D);
+        for (int g = 0; g < per && split * per + g < kGroups8; ++g) {
+          float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < kMaxClusterSplit; ++k) {
+            if (k < ns) {
+              const uint32_t at = data + (uint32_t)((k * per + g) * 8192 + r * 16);
+              const uint4 y0 = ld_shared_v4(at), y1 = ld_shared_v4(at + 4096);
+              const float wk = w[k] * inv_L;
+              a[0] += wk * __uint_as_float(y0.x); a[1] += wk * __uint_as_float(y0.y);
+              a[2] += wk * __uint_as_float(y0.z); a[3] += wk * __uint_as_float(y0.w);
+              a[4] += wk * __uint_as_float(y1.x); a[5] += wk * __uint_as_float(y1.y);
+              a[6] += wk * __uint_as_float(y1.z); a[7] += wk * __uint_as_float(y1.w);
+            }
+          }
+          orow4[split * per + g] = make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]),
+                                              pack_bf16(a[4], a[5]), pack_bf16(a[6], a[7]));
+        }
+        if (p.lse != nullptr && split == 0)
+          p.lse[((size_t)nd.q_index * p.H + h) * p.T + token] = (M + __log2f(L)) * 0.69314718055994531f;
+      }
+    } else if (ns == 1) {
       if (ok) {
         tc_fence_after();
 #pragma unroll
@@ -1237,16 +1340,14 @@ cudaError_t configure_d(int dev) {
   std::lock_guard<std::mutex> lock(mu);
   if (configured[dev]) return cudaSuccess;
   cudaError_t e;
-  for (auto k : {attend_kernel<D, false, false>, attend_kernel<D, true, false>,
-                 attend_kernel<D, true, true>}) {
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-    if (e != cudaSuccess) return e;
-  }
   // setmaxnreg.inc waits until the block's register pool can serve it: a
   // build whose launch register count leaves the split short would never
   // proceed, so such a build is refused here.
-  for (auto k : {attend_kernel<D, false, false>, attend_kernel<D, true, false>,
-                 attend_kernel<D, true, true>}) {
+  for (auto k : {attend_kernel<D, false, false, false>, attend_kernel<D, true, false, false>,
+                 attend_kernel<D, true, true, false>, attend_kernel<D, false, false, true>,
+                 attend_kernel<D, true, false, true>, attend_kernel<D, true, true, true>}) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    if (e != cudaSuccess) return e;
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, k);
     if (e != cudaSuccess) return e;
@@ -1258,6 +1359,22 @@ cudaError_t configure_d(int dev) {
 }
 
 template <int D>
+void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int grid, int cluster,
+                    cudaStream_t s) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3((unsigned)grid, 1, 1);
+  cfg->blockDim = dim3(kThreads, 1, 1);
+  cfg->dynamicSmemBytes = AttnCfg<D>::kSmemBytes;
+  cfg->stream = s;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cluster;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+template <int D>
 cudaError_t launch_d(const AttnParams& p, int grid, cudaStream_t s) {
   using C = AttnCfg<D>;
   int dev = 0;
@@ -1265,13 +1382,47 @@ cudaError_t launch_d(const AttnParams& p, int grid, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   e = configure_d<D>(dev);
   if (e != cudaSuccess) return e;
-  if (p.masked && (p.own_mask != nullptr || p.hist_mask != nullptr))
-    attend_kernel<D, true, true><<<grid, kThreads, C::kSmemBytes, s>>>(p);
+  const bool token = p.masked && (p.own_mask != nullptr || p.hist_mask != nullptr);
+  if (p.cluster) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config<D>(&cfg, &attr, grid, p.n_split, s);
+    return cudaLaunchKernelEx(&cfg, token      ? attend_kernel<D, true, true, true>
+                                    : p.masked ? attend_kernel<D, true, false, true>
+                                               : attend_kernel<D, false, false, true>, p);
+  }
+  if (token)
+    attend_kernel<D, true, true, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
   else if (p.masked)
-    attend_kernel<D, true, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
+    attend_kernel<D, true, false, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
   else
-    attend_kernel<D, false, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
+    attend_kernel<D, false, false, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
   return cudaGetLastError();
+}
+
+// Clusters of `size` CTAs (one CTA per SM) that can be resident at once on the
+// current device, looked up once per device and size.
+template <int D>
+cudaError_t max_clusters_d(int size, int* out) {
+  static std::mutex mu;
+  static int known[64][kMaxClusterSplit + 1] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  e = configure_d<D>(dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  if (known[dev][size] == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config<D>(&cfg, &attr, size, size, nullptr);
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, attend_kernel<D, false, false, true>, &cfg);
+    if (e != cudaSuccess) return e;
+    known[dev][size] = n + 1;
+  }
+  *out = known[dev][size] - 1;
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -1279,6 +1430,13 @@ cudaError_t launch_d(const AttnParams& p, int grid, cudaStream_t s) {
 cudaError_t launch_attend(const AttnParams& p, int head_dim, int grid, cudaStream_t s) {
   if (head_dim == 128) return launch_d<128>(p, grid, s);
   if (head_dim == 64) return launch_d<64>(p, grid, s);
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t attend_max_clusters(int head_dim, int size, int* clusters) {
+  if (size < 2 || size > kMaxClusterSplit) return cudaErrorInvalidValue;
+  if (head_dim == 128) return max_clusters_d<128>(size, clusters);
+  if (head_dim == 64) return max_clusters_d<64>(size, clusters);
   return cudaErrorInvalidValue;
 }
 

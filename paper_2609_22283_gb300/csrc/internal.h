@@ -13,7 +13,8 @@
 namespace sva {
 
 constexpr int kTile = 128;  // query rows per Q tile and key rows per K/V tile
-constexpr int kMaxSplit = 4;  // key-range splits of one work unit
+constexpr int kMaxSplit = 4;  // key-range splits of one work unit, merged through a workspace
+constexpr int kMaxClusterSplit = 8;  // the same, merged inside a thread-block cluster
 constexpr uint64_t kDefaultWaitTimeoutNs = 1000000000ull;  // bounded device waits: 1 s
 constexpr int kMaskWords = 128;  // block-sparse launches: at most 32 * 128 key tiles per node
 
@@ -53,6 +54,7 @@ struct alignas(128) AttnParams {
   int32_t n_split;      // key-range splits per split work unit (1 = no split)
   int32_t n_full;       // units 0..n_full-1 run unsplit (one CTA each); the
                         // rest are split n_split ways (CTAs after them)
+  int32_t cluster;      // 1: the splits of a unit are one cluster (n_full = 0, no workspace)
   float* ws;            // split partials [unit][split][(d + 2) * 256] fp32, or null
   int* ws_count;        // per-unit arrival counters, zero between launches, or null
   uint64_t timeout_ns;
@@ -117,6 +119,8 @@ cudaError_t static_split_scratch(int device, void** ptr);
 
 // Launchers (defined in the .cu files).  They return the launch error.
 cudaError_t launch_attend(const AttnParams& p, int head_dim, int grid, cudaStream_t s);
+// Clusters of `size` attention CTAs that can be resident at once on the current device.
+cudaError_t attend_max_clusters(int head_dim, int size, int* clusters);
 // `max_states`: 1 + the largest n_ctx.
 cudaError_t launch_mask_scan(const ScanParams& p, int n_nodes, int max_states, cudaStream_t s);
 cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s);

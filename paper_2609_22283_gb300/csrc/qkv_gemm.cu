@@ -130,19 +130,6 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   return r;
 }
 
-// The shared::cluster address of the variable at `addr` (a shared::cta
-// address of this CTA) in the CTA of rank `rank` of the cluster.
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n"
-               "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // Arrives once on a barrier of either CTA of the cluster (release at
 // cluster scope: this thread's earlier writes are visible to the waiter).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {

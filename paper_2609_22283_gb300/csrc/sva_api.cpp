@@ -331,6 +331,58 @@ void plan_split(const sva_cache* c, long long units, int min_tiles, long long ca
   }
 }
 
+// What a launch does: units 0..n_full-1 unsplit, the rest n_split ways, merged
+// through the workspace or (cluster) inside clusters of n_split CTAs.
+struct LaunchPlan {
+  long long n_full = 0;
+  int n_split = 1;
+  bool cluster = false;
+};
+
+// plan_split counts waves of key tiles alone; this rule also counts what a CTA
+// costs besides its key tiles (launch, prologue, first loads, epilogue) and
+// what a merge costs, in units of one key tile of a query-tile pair (about
+// 1.2 us): 6 per CTA, 6 for a merge through the workspace (a 4-way split of 16
+// key tiles took 21.5 us, its 4 key tiles and a CTA's fixed part 12.4), 2 for
+// one inside a cluster.  A split that does not pay for them is not made (24
+// units per node x 4 nodes of 12 key tiles: 43 us split three ways over two
+// waves, 26 us unsplit).  Launches whose splits all fit on the GPU at once are
+// split over clusters, down to two key tiles a CTA.
+sva_status plan_launch(const sva_cache* c, long long units, int tiles, long long cap,
+                       LaunchPlan* plan) {
+  const long long sms = c->num_sms;
+  constexpr long long kCta = 6, kMerge = 6, kClusterMerge = 2;
+  auto waves = [&](long long n) { return (n + sms - 1) / sms; };
+  long long n_full = 0;
+  int n_split = 1;
+  plan_split(c, units, tiles, cap, &n_full, &n_split);
+  *plan = LaunchPlan();
+  long long best = waves(units) * (tiles + kCta);
+  if (n_split > 1) {
+    const long long part = (tiles + n_split - 1) / n_split + kCta;
+    const long long cost =
+        n_full / sms * (tiles + kCta) + waves((units - n_full) * n_split) * part + kMerge;
+    if (cost < best) {
+      best = cost;
+      plan->n_full = n_full;
+      plan->n_split = n_split;
+    }
+  }
+  for (int s = 2; cap > 0 && s <= sva::kMaxClusterSplit && units * s <= sms && tiles / s >= 2; ++s) {
+    const long long cost = (tiles + s - 1) / s + kCta + kClusterMerge;
+    if (cost >= best) continue;
+    int clusters = 0;
+    cudaError_t e = sva::attend_max_clusters(c->g.head_dim, s, &clusters);
+    if (e != cudaSuccess) return cuda_fail(e, "attend cluster occupancy");
+    if (units > clusters) continue;
+    best = cost;
+    plan->n_full = 0;
+    plan->n_split = s;
+    plan->cluster = true;
+  }
+  return SVA_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -772,23 +824,34 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
       cap -= items;
     }
   }
-  long long n_full = 0;
-  int n_split = 1;
-  plan_split(c, units, min_tiles, cap, &n_full, &n_split);
+  LaunchPlan plan;
+  st = plan_launch(c, units, min_tiles, cap, &plan);
+  if (st != SVA_OK) return st;
+  const long long n_full = plan.n_full;
+  const int n_split = plan.n_split;
+  const bool use_ws = n_split > 1 && !plan.cluster;
   char* split_base = c->ws;
   size_t counter_bytes = ws_counter_bytes(c);
   if (scratch == Scratch::kStatic) {
     split_base = nullptr;
-    if (n_split > 1) {
-      const long long split_units = units - n_full;
-      counter_bytes = round_up((size_t)split_units * 4, 256);
-      const size_t need = counter_bytes + (size_t)split_units * n_split * ws_item_bytes(c);
+    // The limit of this entry point is stated for the wave-filling split, also
+    // where the launch turns out to need less scratch or none.
+    long long full0 = 0;
+    int split0 = 1;
+    plan_split(c, units, min_tiles, cap, &full0, &split0);
+    if (split0 > 1) {
+      const long long split_units = units - full0;
+      const size_t need = round_up((size_t)split_units * 4, 256) +
+                          (size_t)split_units * split0 * ws_item_bytes(c);
       if (need > sva::kStaticScratchBytes)
         return fail(SVA_ERR_CAPACITY,
                     "this launch splits %lld work units %d ways and needs %zu bytes of scratch; the "
                     "library's static scratch holds %zu bytes (use sva_attend_nodes with a "
                     "workspace for launches this large)",
-                    split_units, n_split, need, sva::kStaticScratchBytes);
+                    split_units, split0, need, sva::kStaticScratchBytes);
+    }
+    if (use_ws) {
+      counter_bytes = round_up((size_t)(units - n_full) * 4, 256);
       void* addr = nullptr;
       cudaError_t e = sva::static_split_scratch(c->device, &addr);
       if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(split scratch)");
@@ -822,7 +885,8 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
   if (scratch != Scratch::kStatic) c->fault_mode = 0;
   p.n_full = (int32_t)n_full;
   p.n_split = n_split;
-  if (n_split > 1) {
+  p.cluster = plan.cluster ? 1 : 0;
+  if (use_ws) {
     p.ws_count = reinterpret_cast<int*>(split_base);
     p.ws = reinterpret_cast<float*>(split_base + counter_bytes);
     if (scratch == Scratch::kStatic) {
