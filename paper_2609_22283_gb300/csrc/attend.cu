@@ -314,8 +314,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   const int split = whole ? 0 : (int)(blockIdx.x - p.n_full) % p.n_split;
   const int unit = whole ? (int)blockIdx.x : p.n_full + (int)(blockIdx.x - p.n_full) / p.n_split;
   const int sunit = unit - p.n_full;     // index among the split units
-  const int qp = unit % p.n_qp;
-  const int rest = unit / p.n_qp;
+  // Or, where frame causality makes the pairs of a node uneven, pair-major with
+  // the longest walks first, so that the short ones fill the gaps at the end.
+  const int pairs = p.H * p.n_nodes;
+  const int qp = p.qp_major ? p.n_qp - 1 - unit / pairs : unit % p.n_qp;
+  const int rest = p.qp_major ? unit % pairs : unit / p.n_qp;
   const int ni = rest % p.n_nodes;
   const int h = rest / p.n_nodes;
   const AttnNode& nd = p.nodes[ni];

@@ -54,6 +54,7 @@ struct alignas(128) AttnParams {
   int32_t n_split;      // key-range splits per split work unit (1 = no split)
   int32_t n_full;       // units 0..n_full-1 run unsplit (one CTA each); the
                         // rest are split n_split ways (CTAs after them)
+  int32_t qp_major;     // 1: units ordered by query-tile pair, the last first, then head and node
   int32_t cluster;      // 1: the splits of a unit are one cluster (n_full = 0, no workspace)
   float* ws;            // split partials [unit][split][(d + 2) * 256] fp32, or null
   int* ws_count;        // per-unit arrival counters, zero between launches, or null

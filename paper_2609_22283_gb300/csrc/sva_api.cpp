@@ -348,8 +348,13 @@ struct LaunchPlan {
 // units per node x 4 nodes of 12 key tiles: 43 us split three ways over two
 // waves, 26 us unsplit).  Launches whose splits all fit on the GPU at once are
 // split over clusters, down to two key tiles a CTA.
-sva_status plan_launch(const sva_cache* c, long long units, int tiles, long long cap,
-                       LaunchPlan* plan) {
+//
+// tiles, max_tiles: the fewest and the most key tiles that a unit walks.  They
+// differ under frame causality (`uneven`: the units are launched longest
+// first, so unsplit ones pack like a sorted list: the mean fills the GPU, and
+// no unit is cut shorter than the longest).
+sva_status plan_launch(const sva_cache* c, long long units, int tiles, int max_tiles, bool uneven,
+                       long long cap, LaunchPlan* plan) {
   const long long sms = c->num_sms;
   constexpr long long kCta = 6, kMerge = 6, kClusterMerge = 2;
   auto waves = [&](long long n) { return (n + sms - 1) / sms; };
@@ -357,11 +362,13 @@ sva_status plan_launch(const sva_cache* c, long long units, int tiles, long long
   int n_split = 1;
   plan_split(c, units, tiles, cap, &n_full, &n_split);
   *plan = LaunchPlan();
-  long long best = waves(units) * (tiles + kCta);
+  const int mean = (tiles + max_tiles) / 2;
+  long long best = waves(units) * (max_tiles + kCta);
+  if (uneven) best = std::max<long long>((units * (mean + kCta) + sms - 1) / sms, max_tiles + kCta);
   if (n_split > 1) {
-    const long long part = (tiles + n_split - 1) / n_split + kCta;
+    const long long part = (mean + n_split - 1) / n_split + kCta;
     const long long cost =
-        n_full / sms * (tiles + kCta) + waves((units - n_full) * n_split) * part + kMerge;
+        n_full / sms * (max_tiles + kCta) + waves((units - n_full) * n_split) * part + kMerge;
     if (cost < best) {
       best = cost;
       plan->n_full = n_full;
@@ -369,7 +376,7 @@ sva_status plan_launch(const sva_cache* c, long long units, int tiles, long long
     }
   }
   for (int s = 2; cap > 0 && s <= sva::kMaxClusterSplit && units * s <= sms && tiles / s >= 2; ++s) {
-    const long long cost = (tiles + s - 1) / s + kCta + kClusterMerge;
+    const long long cost = (max_tiles + s - 1) / s + kCta + kClusterMerge;
     if (cost >= best) continue;
     int clusters = 0;
     cudaError_t e = sva::attend_max_clusters(c->g.head_dim, s, &clusters);
@@ -825,7 +832,24 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
     }
   }
   LaunchPlan plan;
-  st = plan_launch(c, units, min_tiles, cap, &plan);
+  // Pair-major order costs the L2 reuse of a head's K/V by the CTAs that run
+  // together, so it is taken where the pairs differ by more than a quarter and
+  // the launch's K/V (every node's slots, 64 MB of the 129 MB L2) stay in L2
+  // whatever the order.  First chunk of 4680 tokens, 12 heads: 13 to 37 key
+  // tiles a pair, 103 us head-major with the last wave split, 87 us so.
+  int max_tiles = 0;
+  long long kv_rows = 0;
+  for (int i = 0; i < n_nodes; ++i) {
+    max_tiles = std::max(max_tiles, p.nodes[i].n_kv * p.nt_slot);
+    kv_rows += 2LL * p.nodes[i].n_kv * g.num_heads * c->L.Tpad;
+  }
+  bool fc = false;
+  for (int i = 0; i < n_nodes; ++i) fc = fc || p.nodes[i].frame_causal;
+  p.qp_major = fc && (max_tiles - min_tiles) * 4 > max_tiles &&
+                       kv_rows * g.head_dim * 2 <= (64LL << 20)
+                   ? 1
+                   : 0;
+  st = plan_launch(c, units, min_tiles, max_tiles, p.qp_major != 0, cap, &plan);
   if (st != SVA_OK) return st;
   const long long n_full = plan.n_full;
   const int n_split = plan.n_split;
