@@ -112,16 +112,21 @@ __device__ __forceinline__ uint32_t col_o(int b) {
 
 // 12 warps: warpgroup 0 = TMA producer (warp 0), MMA issuers (warps 1 and
 // 3), warp 2 (the block-sparse mask gather in the prologue, then idle);
-// warpgroups 1 and 2 = softmax.  The launch gives every thread
-// kLaunchRegs registers; warpgroup 0 then gives registers back
-// (setmaxnreg.dec to kRegsLow) and the softmax warpgroups take them
-// (setmaxnreg.inc to kRegsHigh).  The split must fit the launch's pool:
-// 4*32*kRegsLow + 8*32*kRegsHigh <= 384*kLaunchRegs, checked at launch.
+// warpgroups 1 and 2 = softmax.  The launch gives every thread kLaunchRegs
+// registers; warpgroup 0 then gives registers back (setmaxnreg.dec to
+// kRegsLow) and the softmax warpgroups take them (setmaxnreg.inc to
+// kRegsHigh).  The split must fit the launch's pool: 4*32*kRegsLow +
+// 8*32*kRegsHigh <= 384*kLaunchRegs, checked at launch.  At D = 64 a softmax
+// thread holds 128 scores and spills below 216 (88 + 208 was 3% slower).
 constexpr int kThreads = 384;
 constexpr int kLaunchRegs = 168;
-constexpr int kRegsLow = 88;
-constexpr int kRegsHigh = 208;
-static_assert(4 * 32 * kRegsLow + 8 * 32 * kRegsHigh <= kThreads * kLaunchRegs, "register split");
+template <int D>
+struct AttnRegs {
+  static constexpr int kLow = D == 128 ? 88 : 72;
+  static constexpr int kHigh = D == 128 ? 208 : 216;
+  static constexpr int kPool = 4 * 32 * kLow + 8 * 32 * kHigh;
+  static_assert(kPool <= kThreads * kLaunchRegs, "register split");
+};
 // Lazy rescale of O: a row's running max m is only moved (and O, l scaled)
 // when a tile's max exceeds it by more than this many log2 units, so P =
 // 2^(x - m) <= 2^64 between rescales.  Then l <= 2^(64 + 16) for up to 2^16
@@ -309,18 +314,22 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   // The first n_full units run unsplit (one CTA each, the full waves); the
   // others are split n_split ways, the splits of a unit adjacent.
   // kCluster: one cluster of n_split CTAs per unit (n_full = 0).
-  const bool whole = !kCluster && (int)blockIdx.x < p.n_full;
-  const int ns = whole ? 1 : p.n_split;  // key ranges of this unit
-  const int split = whole ? 0 : (int)(blockIdx.x - p.n_full) % p.n_split;
-  const int unit = whole ? (int)blockIdx.x : p.n_full + (int)(blockIdx.x - p.n_full) / p.n_split;
+  int ns = 1, split = 0, unit = (int)blockIdx.x;  // key ranges of the unit, this CTA's
+  if (kCluster || unit >= p.n_full) {
+    ns = p.n_split;
+    const uint32_t rem = blockIdx.x - (uint32_t)p.n_full, u = rem / (uint32_t)ns;
+    split = (int)(rem - u * (uint32_t)ns);
+    unit = p.n_full + (int)u;
+  }
   const int sunit = unit - p.n_full;     // index among the split units
   // Or, where frame causality makes the pairs of a node uneven, pair-major with
   // the longest walks first, so that the short ones fill the gaps at the end.
-  const int pairs = p.H * p.n_nodes;
-  const int qp = p.qp_major ? p.n_qp - 1 - unit / pairs : unit % p.n_qp;
-  const int rest = p.qp_major ? unit % pairs : unit / p.n_qp;
-  const int ni = rest % p.n_nodes;
-  const int h = rest / p.n_nodes;
+  const uint32_t by = (uint32_t)(p.qp_major ? p.H * p.n_nodes : p.n_qp);
+  const uint32_t major = (uint32_t)unit / by, minor = (uint32_t)unit - major * by;
+  const int qp = p.qp_major ? p.n_qp - 1 - (int)major : (int)minor;
+  const uint32_t rest = p.qp_major ? minor : major;
+  const int h = (int)(rest / (uint32_t)p.n_nodes);
+  const int ni = (int)rest - h * p.n_nodes;
   const AttnNode& nd = p.nodes[ni];
   const int n_all = nd.n_kv * p.nt_slot;  // key tiles of the node
   const int qt0 = 2 * qp;
@@ -342,14 +351,33 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   // tiles either query tile may attend (set in the prologue below).
   constexpr bool sparse = kSparse;  // a launch with a block-sparse tile mask
   const int n_eff = n_all - (gap_hi - gap_lo);
-  int t_begin = (int)((long long)split * n_eff / ns);
-  int n_tiles = (int)((long long)(split + 1) * n_eff / ns) - t_begin;
+  int t_begin = 0, n_tiles = n_eff;
+  if (ns > 1) {
+    t_begin = split * n_eff / ns;
+    n_tiles = (split + 1) * n_eff / ns - t_begin;
+  }
   if (t_begin >= gap_lo) t_begin += gap_hi - gap_lo;
   // per query tile, bit i = kernel key tile i (block-sparse instances only)
   __shared__ uint32_t tmask[2][kSparse ? kMaskWords : 1];
   __shared__ int sp_first, sp_count;
 
+  uint8_t* sQ0 = smem + C::kOffQ0;
+  uint8_t* sQ1 = smem + C::kOffQ1;
+  uint8_t* sK = smem + C::kOffK;
+  uint8_t* sV = smem + C::kOffV;
+  auto load_q = [&]() {
+    mbar_arrive_expect_tx(&bars.q_full, (has_q1 ? 2 : 1) * C::kTileBytes);
+#pragma unroll
+    for (int b = 0; b < C::kBoxes; ++b) {
+      tma_load_4d(sQ0 + b * C::kBoxBytes, &p.tmap_q, &bars.q_full, b * 64, h, qt0 * kTile, nd.q_index);
+      if (has_q1)
+        tma_load_4d(sQ1 + b * C::kBoxBytes, &p.tmap_q, &bars.q_full, b * 64, h, (qt0 + 1) * kTile,
+                    nd.q_index);
+    }
+  };
   if (threadIdx.x == 0) {
+    prefetch_tmap(&p.tmap_q);
+    prefetch_tmap(&p.tmap_kv);
     abort_flag = 0;
     mbar_init(&bars.q_full, 1);
     mbar_init(&bars.o_final, 2);  // one commit per MMA issuer
@@ -367,6 +395,21 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       mbar_init(&bars.v_empty[s], C::kOwnTile && has_q1 ? 2 : 1);
     }
     fence_mbar_init();
+    if constexpr (!sparse) {
+      // Q and the first K tile are on their way while the CTA sets up the
+      // rest: they used to follow the set-up, 600 cycles later.
+      fence_proxy_async_smem();
+      load_q();
+      if (n_tiles > 0) {
+        const int st = t_begin / p.nt_slot;
+        const int row_k = (nd.slot[st] * 2 * p.H + h) * p.Tpad + (t_begin - st * p.nt_slot) * kTile;
+        const uint64_t keep = l2_policy_evict_last();
+        mbar_arrive_expect_tx(&bars.k_full[0], C::kTileBytes);
+#pragma unroll
+        for (int b = 0; b < C::kBoxes; ++b)
+          tma_load_2d_hint(sK + b * C::kBoxBytes, &p.tmap_kv, &bars.k_full[0], b * 64, row_k, keep);
+      }
+    }
   }
   if (warp == 1) {
     tmem_alloc(&tmem_base_sh, C::kTmemCols);
@@ -434,28 +477,14 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   const uint32_t tbase = tmem_base_sh;
   const uint64_t tmo = p.timeout_ns;
 
-  uint8_t* sQ0 = smem + C::kOffQ0;
-  uint8_t* sQ1 = smem + C::kOffQ1;
-  uint8_t* sK = smem + C::kOffK;
-  uint8_t* sV = smem + C::kOffV;
   int k_issued = 0, v_issued = 0;  // producer: tiles whose K / V copies were started
 
   if (warp < 4) {
-    regs_dec<kRegsLow>();
+    regs_dec<AttnRegs<D>::kLow>();
     if (warp == 0) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
-      prefetch_tmap(&p.tmap_q);
-      prefetch_tmap(&p.tmap_kv);
-      mbar_arrive_expect_tx(&bars.q_full, (has_q1 ? 2 : 1) * C::kTileBytes);
-#pragma unroll
-      for (int b = 0; b < C::kBoxes; ++b) {
-        tma_load_4d(sQ0 + b * C::kBoxBytes, &p.tmap_q, &bars.q_full, b * 64, h, qt0 * kTile,
-                    nd.q_index);
-        if (has_q1)
-          tma_load_4d(sQ1 + b * C::kBoxBytes, &p.tmap_q, &bars.q_full, b * 64, h,
-                      (qt0 + 1) * kTile, nd.q_index);
-      }
+      if constexpr (sparse) load_q();
       const uint64_t keep = l2_policy_evict_last();
       TileWalk<kSparse ? kMaskWords : 1> walk;
       if constexpr (sparse) walk.start(tmask, t_begin, n_all);
@@ -467,16 +496,18 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         const int t = i - (i / p.nt_slot) * p.nt_slot;
         const int row_k = ((slot * 2 + 0) * p.H + h) * p.Tpad + t * kTile;
         const int row_v = row_k + p.H * p.Tpad;
-        if (!mbar_wait(&bars.k_empty[ks], ((uint32_t)(j / C::kKStages) & 1u) ^ 1u, &abort_flag,
-                       tmo)) {
-          record_timeout(p, &abort_flag);
-          break;
-        }
-        mbar_arrive_expect_tx(&bars.k_full[ks], C::kTileBytes);
+        if (sparse || j > 0) {  // a dense walk's first K tile is on its way already
+          if (!mbar_wait(&bars.k_empty[ks], ((uint32_t)(j / C::kKStages) & 1u) ^ 1u, &abort_flag,
+                         tmo)) {
+            record_timeout(p, &abort_flag);
+            break;
+          }
+          mbar_arrive_expect_tx(&bars.k_full[ks], C::kTileBytes);
 #pragma unroll
-        for (int b = 0; b < C::kBoxes; ++b)
-          tma_load_2d_hint(sK + ks * C::kTileBytes + b * C::kBoxBytes, &p.tmap_kv,
-                           &bars.k_full[ks], b * 64, row_k, keep);
+          for (int b = 0; b < C::kBoxes; ++b)
+            tma_load_2d_hint(sK + ks * C::kTileBytes + b * C::kBoxBytes, &p.tmap_kv,
+                             &bars.k_full[ks], b * 64, row_k, keep);
+        }
         k_issued = j + 1;
         if (!mbar_wait(&bars.v_empty[vs], ((uint32_t)(j / C::kVStages) & 1u) ^ 1u, &abort_flag,
                        tmo)) {
@@ -695,7 +726,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       tmem_dealloc(tbase, C::kTmemCols);
     }
   } else {
-    regs_inc<kRegsHigh>();
+    regs_inc<AttnRegs<D>::kHigh>();
     // ------------------------------------------------------------ softmax + epilogue
     // D = 128: all eight softmax warps work on one query tile at a time (tile
     // 0, then tile 1, of every key tile).  A warp covers 16 rows, half of its
@@ -1179,6 +1210,13 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           p.lse[((size_t)nd.q_index * p.H + h) * p.T + token] = (M + __log2f(L)) * 0.69314718055994531f;
       }
     } else if (ns == 1) {
+      // Each thread's row of O goes to the shared memory of its Q tile (no
+      // longer needed; the 128-byte swizzle keeps the writes free of bank
+      // conflicts), and the warp stores its rows whole: 256 or 128 contiguous
+      // bytes a row, 512 a warp instruction.  Stores straight from the threads
+      // touched 32 lines an instruction and took 6700 cycles a CTA; TMA tile
+      // stores 3700, 2100 of them waiting for the copy to read 64 KB of shared
+      // memory before the CTA may leave; these 3250.
       if (ok) {
         tc_fence_after();
 #pragma unroll
@@ -1186,9 +1224,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           const int b = C::kOwnTile ? b_own : x;
           if (b >= nb) break;
           const int token = (qt0 + b) * kTile + row;
-          const bool in_range = token < p.T;
-          __nv_bfloat16* orow = static_cast<__nv_bfloat16*>(p.out) +
-                                (((size_t)nd.q_index * p.T + token) * p.H + h) * D + DH * half;
+          const uint32_t srow = smem_u32(b ? sQ1 : sQ0) + (uint32_t)(half * C::kBoxBytes + row * 128);
           const float inv_l = l_row[x] > 0.0f ? 1.0f / l_row[x] : 0.0f;  // no visible key: O = 0
 #pragma unroll
           for (int c = 0; c < DH / 32; ++c) {
@@ -1199,22 +1235,39 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 #pragma unroll
               for (int e = 0; e < 32; ++e) o[e] = 0u;
             }
-            if (in_range) {
-              uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
 #pragma unroll
-              for (int v = 0; v < 4; ++v) {
-                uint4 w;
-                w.x = pack_bf16(__uint_as_float(o[v * 8 + 0]) * inv_l, __uint_as_float(o[v * 8 + 1]) * inv_l);
-                w.y = pack_bf16(__uint_as_float(o[v * 8 + 2]) * inv_l, __uint_as_float(o[v * 8 + 3]) * inv_l);
-                w.z = pack_bf16(__uint_as_float(o[v * 8 + 4]) * inv_l, __uint_as_float(o[v * 8 + 5]) * inv_l);
-                w.w = pack_bf16(__uint_as_float(o[v * 8 + 6]) * inv_l, __uint_as_float(o[v * 8 + 7]) * inv_l);
-                dst[v] = w;
-              }
+            for (int v = 0; v < 4; ++v) {
+              uint32_t w[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                w[e] = pack_bf16(__uint_as_float(o[v * 8 + 2 * e]) * inv_l,
+                                 __uint_as_float(o[v * 8 + 2 * e + 1]) * inv_l);
+              st_shared_v4(srow + (uint32_t)(((c * 4 + v) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
             }
           }
-          if (p.lse != nullptr && in_range && half == 0)
+          if (p.lse != nullptr && token < p.T && half == 0)
             p.lse[((size_t)nd.q_index * p.H + h) * p.T + token] =
                 (m[x] + __log2f(l_row[x])) * 0.69314718055994531f;
+        }
+        __syncwarp();
+        constexpr int kPieces = D / 8;                     // 16-byte pieces of a row
+        constexpr int kRows = 32 / C::kRowThreads;         // rows of this warp per query tile
+        const int r0 = row - (C::kOwnTile ? lane : lane & 15);
+        const int piece = lane % kPieces;
+#pragma unroll
+        for (int x = 0; x < NT; ++x) {
+          const int b = C::kOwnTile ? b_own : x;
+          if (b >= nb) break;
+          const uint32_t box = smem_u32(b ? sQ1 : sQ0) + (uint32_t)((piece >> 3) * C::kBoxBytes);
+          __nv_bfloat16* o0 = static_cast<__nv_bfloat16*>(p.out) +
+                              (((size_t)nd.q_index * p.T + (qt0 + b) * kTile) * p.H + h) * D + piece * 8;
+#pragma unroll
+          for (int k = 0; k < kRows * kPieces / 32; ++k) {
+            const int r = r0 + k * (32 / kPieces) + lane / kPieces;
+            const uint4 v = ld_shared_v4(box + (uint32_t)(r * 128 + (((piece & 7) ^ (r & 7)) << 4)));
+            if ((qt0 + b) * kTile + r < p.T)
+              *reinterpret_cast<uint4*>(o0 + (size_t)r * p.H * D) = v;
+          }
         }
       }
     } else {
@@ -1354,7 +1407,7 @@ cudaError_t configure_d(int dev) {
     cudaFuncAttributes fa;
     e = cudaFuncGetAttributes(&fa, k);
     if (e != cudaSuccess) return e;
-    if (fa.numRegs * kThreads < 4 * 32 * kRegsLow + 8 * 32 * kRegsHigh)
+    if (fa.numRegs * kThreads < AttnRegs<D>::kPool)
       return cudaErrorInvalidConfiguration;
   }
   configured[dev] = true;
