@@ -67,13 +67,13 @@ __device__ __forceinline__ uint32_t rotate_pair(uint32_t xy, float c, float s) {
 // token-major inputs, so the warp walks them as 16-byte vectors; lane l always
 // holds vector l mod (d/8) of a head row, i.e. the same four pairs for every
 // head, so its cos/sin come from the tables once per token.
-// Instances: with the RMSNorm of K (and Q), and two without it.  kWave
+// Two instances (the RMSNorm of K and Q has a kernel of its own).  kWave
 // holds the kernel to 64 registers (loads in batches of two), so four
 // 256-thread blocks fit an SM and a launch of one 4680-token node (585
 // blocks) runs in a single wave: such a launch is bound by memory latency,
 // and occupancy is what hides it.  Larger launches loop over their tokens
 // and do better with batches of four at two blocks per SM.
-template <bool kNorm, bool kWave>
+template <bool kWave>
 __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __grid_constant__ RopeParams p) {
   const int lane = threadIdx.x & 31;
   const int vpr = p.d >> 3;                        // 16-byte vectors per (token, head) row
@@ -112,26 +112,6 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
     }
     const size_t in_tok = (size_t)tok * per_tok * 8;
     const size_t out_slot = ((size_t)nd.slot * 2 * p.H) * p.Tpad;  // row of (slot, K, head 0)
-    // RMSNorm scale of the token's K and Q vectors (pass over the row, then a
-    // warp reduction); the second pass below reloads the row from L1/L2.
-    float rk = 1.0f, rq = 1.0f;
-    constexpr bool norm = kNorm;
-    if constexpr (norm) {
-      float sk = 0.0f, sq = 0.0f;
-      for (int v = lane; v < per_tok; v += 32) {
-        const size_t off = in_tok + (size_t)v * 8;
-        sk += sumsq8(*reinterpret_cast<const uint4*>(kin + off));
-        if (qio) sq += sumsq8(*reinterpret_cast<const uint4*>(qio + off));
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        sk += __shfl_xor_sync(0xffffffffu, sk, o);
-        sq += __shfl_xor_sync(0xffffffffu, sq, o);
-      }
-      const float inv_n = 1.0f / (float)(per_tok * 8);
-      rk = __frsqrt_rn(__fmaf_rn(sk, inv_n, p.norm_eps));
-      rq = __frsqrt_rn(__fmaf_rn(sq, inv_n, p.norm_eps));
-    }
     // Batches of kBatch vectors per lane: every load of a batch is issued
     // before any of its stores (q is rotated in place, so without the split
     // the compiler keeps each iteration's loads behind the previous stores).
@@ -158,28 +138,10 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
         const size_t in_off = in_tok + (size_t)v * 8;
         uint32_t kw[4] = {kv[j].x, kv[j].y, kv[j].z, kv[j].w};
         uint32_t qw[4] = {qv[j].x, qv[j].y, qv[j].z, qv[j].w};
-        if constexpr (norm) {
-          const float4* gk = reinterpret_cast<const float4*>(p.gamma_k + (size_t)v * 8);
-          const float4 gk0 = __ldg(gk), gk1 = __ldg(gk + 1);
-          const float gkk[8] = {gk0.x, gk0.y, gk0.z, gk0.w, gk1.x, gk1.y, gk1.z, gk1.w};
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            kw[k] = norm_rotate_pair(kw[k], gkk[2 * k] * rk, gkk[2 * k + 1] * rk, cs[k].x, cs[k].y);
-          if (qio) {
-            const float4* gq = reinterpret_cast<const float4*>(p.gamma_q + (size_t)v * 8);
-            const float4 gq0 = __ldg(gq), gq1 = __ldg(gq + 1);
-            const float gqq[8] = {gq0.x, gq0.y, gq0.z, gq0.w, gq1.x, gq1.y, gq1.z, gq1.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              qw[k] = norm_rotate_pair(qw[k], gqq[2 * k] * rq, gqq[2 * k + 1] * rq, cs[k].x,
-                                       cs[k].y);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            kw[k] = rotate_pair(kw[k], cs[k].x, cs[k].y);
-            qw[k] = rotate_pair(qw[k], cs[k].x, cs[k].y);
-          }
+        for (int k = 0; k < 4; ++k) {
+          kw[k] = rotate_pair(kw[k], cs[k].x, cs[k].y);
+          qw[k] = rotate_pair(qw[k], cs[k].x, cs[k].y);
         }
         __nv_bfloat16* kdst = cache + ((out_slot + (size_t)h * p.Tpad + u) * p.d + c8 * 8);
         *reinterpret_cast<uint4*>(kdst) = make_uint4(kw[0], kw[1], kw[2], kw[3]);
@@ -190,16 +152,165 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
   }
 }
 
+// The same with an RMSNorm of the token's K (and Q) vector of H*d elements in
+// front of the rotation.  kWarps warps share a token and keep its K and Q in
+// registers (at most kVec 16-byte vectors a lane and tensor) from the sum of
+// squares to the rotation, so every input is read once; V is stored once the
+// sums are reduced (shuffles, then shared memory across the token's warps).
+// One block of eight warps takes 8 / kWarps tokens, all their loads in flight
+// at once; two or three blocks an SM (registers) is what its bandwidth needs:
+// one block gave 4.6 TB/s where two give 6.3, and fewer registers spill.
+// Against reading the rows twice with one warp a token (all with CUDA graphs,
+// three sets of buffers): 4680 tokens x 40 x 128, K and V (192 MB) 37.9 -> 35.0
+// us; 4 x 4680 tokens x 12 x 128 with Q (345 MB) 68.7 -> 58.7 us, x 40 x 128
+// (1150 MB) 204 -> 183 us; one node of 12 x 128 with Q 19.5 -> 19.4 us (a
+// device copy of its 43 MB takes 20.5 us in the same loop).
+template <int kWarps, int kVec, bool kQ>
+__global__ void __launch_bounds__(256, kVec <= 3 || !kQ ? 3 : 2)
+    rope_norm_kernel(const __grid_constant__ RopeParams p) {
+  __shared__ float part[8][2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int vpr = p.d >> 3;                        // 16-byte vectors per (token, head) row
+  const int vshift = (vpr == 16) ? 4 : 3;
+  const int c8 = lane & (vpr - 1);
+  const int per_tok = p.H * vpr;                   // vectors per token
+  const int tok = blockIdx.x * (8 / kWarps) + warp / kWarps;
+  const bool live = tok < p.n_nodes * p.T;         // the last block may have tokens to spare
+  const __nv_bfloat16* kin = static_cast<const __nv_bfloat16*>(p.k_new);
+  const __nv_bfloat16* vin = static_cast<const __nv_bfloat16*>(p.v_new);
+  __nv_bfloat16* qio = static_cast<__nv_bfloat16*>(p.q);
+  __nv_bfloat16* cache = static_cast<__nv_bfloat16*>(p.cache);
+  const size_t kv_stride = (size_t)p.H * p.Tpad * p.d;  // elements between K and V of a slot
+  const int v0 = (warp % kWarps) * 32 + lane;
+  const size_t in_tok = (size_t)tok * per_tok * 8;
+  uint4 kv[kVec], qv[kQ ? kVec : 1], vv[kVec];
+#pragma unroll
+  for (int j = 0; j < kVec; ++j) {
+    const int v = v0 + j * 32 * kWarps;
+    const bool in = live && v < per_tok;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    kv[j] = in ? ld_stream(kin + in_tok + (size_t)v * 8) : zero;
+    if constexpr (kQ) qv[j] = in ? *reinterpret_cast<const uint4*>(qio + in_tok + (size_t)v * 8) : zero;
+    vv[j] = in ? ld_stream(vin + in_tok + (size_t)v * 8) : zero;
+  }
+  const int HpWp = p.Hp * p.Wp;
+  const int node = live ? tok / p.T : 0;
+  const int u = live ? tok - node * p.T : 0;
+  const int f = u / HpWp;
+  const int hw = u - f * HpWp;
+  const int hh = hw / p.Wp;
+  const int ww = hw - hh * p.Wp;
+  const RopeNode nd = p.nodes[node];
+  const int tpos = nd.t_base + f;
+  float2 cs[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int pi = c8 * 4 + k;  // pair index within the head dimension
+    if (pi < p.P0)
+      cs[k] = __ldg(p.tab_t + (size_t)tpos * p.P0 + pi);
+    else if (pi < p.P0 + p.P1)
+      cs[k] = __ldg(p.tab_h + (size_t)hh * p.P1 + (pi - p.P0));
+    else
+      cs[k] = __ldg(p.tab_w + (size_t)ww * p.P2 + (pi - p.P0 - p.P1));
+  }
+  const size_t out_slot = ((size_t)nd.slot * 2 * p.H) * p.Tpad;  // row of (slot, K, head 0)
+  auto cache_at = [&](int v) {
+    return cache + ((out_slot + (size_t)(v >> vshift) * p.Tpad + u) * p.d + c8 * 8);
+  };
+  float sk = 0.0f, sq = 0.0f;
+#pragma unroll
+  for (int j = 0; j < kVec; ++j) {
+    sk += sumsq8(kv[j]);
+    if constexpr (kQ) sq += sumsq8(qv[j]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sk += __shfl_xor_sync(0xffffffffu, sk, o);
+    sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  }
+  if constexpr (kWarps > 1) {
+    if (lane == 0) {
+      part[warp][0] = sk;
+      part[warp][1] = sq;
+    }
+    __syncthreads();
+    sk = 0.0f;
+    sq = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      sk += part[warp / kWarps * kWarps + w][0];
+      sq += part[warp / kWarps * kWarps + w][1];
+    }
+  }
+  if (!live) return;
+#pragma unroll
+  for (int j = 0; j < kVec; ++j) {
+    const int v = v0 + j * 32 * kWarps;
+    if (v < per_tok) *reinterpret_cast<uint4*>(cache_at(v) + kv_stride) = vv[j];
+  }
+  const float inv_n = 1.0f / (float)(per_tok * 8);
+  const float rk = __frsqrt_rn(__fmaf_rn(sk, inv_n, p.norm_eps));
+  const float rq = __frsqrt_rn(__fmaf_rn(sq, inv_n, p.norm_eps));
+  // x * gamma / rms of one vector, rotated
+  auto norm_rotate = [&](uint4 x, const float* gamma, int v, float r) {
+    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gamma + (size_t)v * 8));
+    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gamma + (size_t)v * 8) + 1);
+    return make_uint4(norm_rotate_pair(x.x, g0.x * r, g0.y * r, cs[0].x, cs[0].y),
+                      norm_rotate_pair(x.y, g0.z * r, g0.w * r, cs[1].x, cs[1].y),
+                      norm_rotate_pair(x.z, g1.x * r, g1.y * r, cs[2].x, cs[2].y),
+                      norm_rotate_pair(x.w, g1.z * r, g1.w * r, cs[3].x, cs[3].y));
+  };
+#pragma unroll
+  for (int j = 0; j < kVec; ++j) {
+    const int v = v0 + j * 32 * kWarps;
+    if (v < per_tok) {
+      *reinterpret_cast<uint4*>(cache_at(v)) = norm_rotate(kv[j], p.gamma_k, v, rk);
+      if constexpr (kQ)
+        *reinterpret_cast<uint4*>(qio + in_tok + (size_t)v * 8) = norm_rotate(qv[j], p.gamma_q, v, rq);
+    }
+  }
+}
+
+template <int kWarps, int kVec>
+void launch_norm(const RopeParams& p, cudaStream_t s) {
+  const long long tokens = (long long)p.n_nodes * p.T;
+  constexpr int per_block = 8 / kWarps;
+  const unsigned grid = (unsigned)((tokens + per_block - 1) / per_block);
+  if (p.q != nullptr)
+    rope_norm_kernel<kWarps, kVec, true><<<grid, 256, 0, s>>>(p);
+  else
+    rope_norm_kernel<kWarps, kVec, false><<<grid, 256, 0, s>>>(p);
+}
+
 }  // namespace
 
 cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s) {
   const long long blocks = ((long long)p.n_nodes * p.T + 7) / 8;  // one warp per token
-  if (p.gamma_k != nullptr)
-    rope_kv_kernel<true, false><<<p.grid_blocks, 256, 0, s>>>(p);
-  else if (blocks <= 4LL * num_sms)
-    rope_kv_kernel<false, true><<<p.grid_blocks, 256, 0, s>>>(p);
-  else
-    rope_kv_kernel<false, false><<<p.grid_blocks, 256, 0, s>>>(p);
+  const int per_tok = p.H * (p.d >> 3);  // 16-byte vectors, at most 2048
+  if (p.gamma_k != nullptr) {
+    // Few vectors a lane where that costs no bandwidth (a small launch is as
+    // long as one token takes: 320 tokens of 12 x 128, 5.4 us at six vectors,
+    // 4.0 at three), more where three would leave warps short of loads (40 x
+    // 128: 38 us at three, 35 at five; 16 x 64: 13.5 at three, 12.6 at four).
+    if (per_tok <= 64)
+      launch_norm<1, 2>(p, s);
+    else if (per_tok <= 128)
+      launch_norm<1, 4>(p, s);
+    else if (per_tok <= 192)
+      launch_norm<2, 3>(p, s);
+    else if (per_tok <= 384)
+      launch_norm<4, 3>(p, s);
+    else if (per_tok <= 640)
+      launch_norm<4, 5>(p, s);
+    else if (per_tok <= 1280)
+      launch_norm<8, 5>(p, s);
+    else
+      launch_norm<8, 8>(p, s);
+  } else if (blocks <= 4LL * num_sms) {
+    rope_kv_kernel<true><<<p.grid_blocks, 256, 0, s>>>(p);
+  } else {
+    rope_kv_kernel<false><<<p.grid_blocks, 256, 0, s>>>(p);
+  }
   return cudaGetLastError();
 }
 

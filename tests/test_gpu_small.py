@@ -7,7 +7,7 @@ rescale threshold in mid-sequence.
 
 Reference: the same op in fp64 torch on the rotated Q and the K', V the cache
 holds.  Bound per element: the rounding of P to bf16 moves O by at most
-2^-8 E_p|V|, that of the output by at most 2^-9 |O|, and fp32 logits of size
+2^-8 E_p|V|, that of the output by at most 2^-8 |O|, and fp32 logits of size
 L carry an error of about 2^-22 L (L < 2^11 log2 units here, so 2^-11), which
 scales the weights: |d| <= 2^-8 (E_p|V| + |O|) + 2^-10 E_p|V|, and 2^-20 for
 the fp32 sums themselves (|V| < 8), which is all that is left where a row's
