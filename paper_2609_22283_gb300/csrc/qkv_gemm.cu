@@ -29,7 +29,7 @@
 // not fit in L2.  When the tiles do not fill the last round of pairs, the
 // tiles of that round are split into two half-width items (BN / 2 columns),
 // so that the last round takes half as long.
-//   warp 0      TMA producer (x and W tiles, 128-byte swizzle);
+//   warps 0, 2  TMA producers (x and W tiles, 128-byte swizzle);
 //   warp 1      TMEM owner (both CTAs) and MMA issuer (even CTA; whole warp,
 //               one elected lane);
 //   warps 4-11  epilogue: two warps per TMEM lane quarter, one output row per
@@ -140,11 +140,11 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 // tma_load_2d whose completion is counted on a barrier that may belong to
 // the peer CTA of the pair (`bar` is a shared::cluster address); the data
 // lands in this CTA's shared memory.
-__device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, uint32_t bar,
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                                  int32_t c0, int32_t c1) {
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
+      " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
       : "memory");
 }
@@ -167,30 +167,52 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
                : "memory");
 }
 
-// D[tmem of both CTAs] (+)= A[smem of both] * B[smem of both], M = 256 rows
-// (128 per CTA); issued by the even CTA only, warp-wide with one elected lane.
-__device__ __forceinline__ void mma_ss_pair_warp(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                                 uint32_t idesc, uint32_t accumulate) {
+// Four MMAs over 64 elements of K: D[tmem of both CTAs] (+)= A[smem of both] *
+// B[smem of both], M = 256 rows (128 per CTA); issued by the even CTA only,
+// warp-wide under one election.  The descriptors advance by 32 bytes of K; the
+// first MMA accumulates where `accumulate` says.
+__device__ __forceinline__ void mma_ss_pair_warp_x4(uint32_t d_tmem, uint64_t a_desc,
+                                                    uint64_t b_desc, uint32_t idesc,
+                                                    uint32_t accumulate) {
   asm volatile(
       "{\n"
-      " .reg .pred p, e;\n"
-      " setp.ne.b32 p, %4, 0;\n"
+      " .reg .pred p, t, e;\n"
+      " setp.ne.b32 p, %10, 0;\n"
+      " setp.eq.b32 t, 0, 0;\n"
       " elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %5, %9, p;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %2, %6, %9, t;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %3, %7, %9, t;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %4, %8, %9, t;\n"
       "}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "l"(a_desc), "l"(a_desc + 2), "l"(a_desc + 4), "l"(a_desc + 6), "l"(b_desc),
+      "l"(b_desc + 2), "l"(b_desc + 4), "l"(b_desc + 6), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
-// Arrives once on the barrier at shared::cluster address `bar` (this CTA's
-// or the peer's) when every tcgen05 operation this thread issued so far has
-// completed; warp-wide, one elected lane.
+// Arrives once on the barrier at shared::cluster address `bar` when every
+// tcgen05 operation this thread issued so far has completed; warp-wide, one
+// elected lane.
 __device__ __forceinline__ void mma_commit_pair_warp(uint32_t bar) {
   asm volatile(
       "{\n"
       " .reg .pred e;\n"
       " elect.sync _|e, 0xffffffff;\n"
       " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+      "}\n" ::"r"(bar)
+      : "memory");
+}
+
+// The same, arriving on the barrier at this offset in both CTAs of the pair.
+__device__ __forceinline__ void mma_commit_both_warp(uint32_t bar) {
+  asm volatile(
+      "{\n"
+      " .reg .pred e;\n"
+      " .reg .b16 m;\n"
+      " mov.b16 m, 3;\n"
+      " elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], m;\n"
       "}\n" ::"r"(bar)
       : "memory");
 }
@@ -244,6 +266,9 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
   const int n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
+    prefetch_tmap(&p.tmap_x);
+    prefetch_tmap(&p.tmap_w);
+    prefetch_tmap(&p.tmap_wh);
     abort_flag = 0;
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&bars.full[s], 1);
@@ -268,35 +293,50 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
   const uint64_t tmo = p.timeout_ns;
   int issued = 0;  // producer: K blocks whose copies were started
 
-  if (warp == 0) {
-    // ------------------------------------------------------------ producer
+  if (warp == 0 || warp == 2) {
+    // ------------------------------------------------------------ producers
+    // x: warp 0, W: warp 2.  A K block took one thread for both 480 cycles, as
+    // long as the MMAs of a whole tile and twice those of a half-width one, so
+    // launches of half-width items were bound by it; a wait on a barrier that
+    // is complete costs about 150 of them.  With two producers, the next
+    // stage's barrier tested while a copy is issued, and the MMA warp issuing
+    // a K block under one election with one commit for both CTAs: 320 rows x
+    // 1536 -> 4608 11.1 -> 10.0 us, 500 x 2048 -> 768 12.2 -> 10.6, 4680 x 1536
+    // 40.0 -> 39.6; where whole tiles fill the GPU, unchanged.
     if (lane == 0) {
-      prefetch_tmap(&p.tmap_x);
-      prefetch_tmap(&p.tmap_w);
-      prefetch_tmap(&p.tmap_wh);
+      const bool is_x = warp == 0;
+      const bool counts = is_x && rank == 0;
       const uint32_t full0 = mapa_shared(smem_u32(&bars.full[0]), 0);  // even CTA's barriers
+      const uint32_t dst = smem_u32(smem) + (is_x ? 0u : (uint32_t)C::kABytes);
+      int s = 0;         // stage and the phase that its barrier has to have left
+      uint32_t ph = 1u;
+      bool ready = true;  // nothing has been loaded yet
       for (int i = pair; i < p.n_items; i += n_pairs) {
         const Item it = item_of(p, i);
         const bool half = it.half >= 0;
         // this CTA's part of the stage: its 128 x rows and its half of the W rows
         const uint32_t bytes = C::kABytes + (half ? C::kBBytes / 2 : C::kBBytes);
-        const int x_row = it.m * 2 * kBM + (int)rank * kBM;
-        const int w_row = it.n * BN + (half ? it.half * (BN / 2) + (int)rank * (BN / 4)
-                                            : (int)rank * (BN / 2));
+        const int row = is_x ? it.m * 2 * kBM + (int)rank * kBM
+                             : it.n * BN + (half ? it.half * (BN / 2) + (int)rank * (BN / 4)
+                                                 : (int)rank * (BN / 2));
+        const CUtensorMap* map = is_x ? &p.tmap_x : (half ? &p.tmap_wh : &p.tmap_w);
         bool ok = true;
         for (int kb = 0; kb < p.n_kblocks; ++kb, ++issued) {
-          const int s = issued % kStages;
-          const uint32_t ph = (uint32_t)(issued / kStages) & 1u;
-          if (!mbar_wait(&bars.empty[s], ph ^ 1u, &abort_flag, tmo)) {
+          if (!ready && !mbar_wait(&bars.empty[s], ph, &abort_flag, tmo)) {
             proj_timeout(p, &abort_flag);
             ok = false;
             break;
           }
-          uint8_t* sa = smem + s * C::kStageBytes;
-          const uint32_t full = full0 + (uint32_t)(s * sizeof(uint64_t));
-          if (rank == 0) mbar_arrive_expect_tx(&bars.full[s], 2 * bytes);  // both CTAs' bytes
-          tma_load_2d_pair(sa, &p.tmap_x, full, kb * kBK, x_row);
-          tma_load_2d_pair(sa + C::kABytes, half ? &p.tmap_wh : &p.tmap_w, full, kb * kBK, w_row);
+          // both CTAs' bytes of x and W (W's may land before this is counted)
+          if (counts) mbar_arrive_expect_tx(&bars.full[s], 2 * bytes);
+          tma_load_2d_pair(dst + (uint32_t)(s * C::kStageBytes), map,
+                           full0 + (uint32_t)(s * sizeof(uint64_t)), kb * kBK, row);
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+          // the next stage's test is on its way while the copy is issued
+          ready = mbar_test_wait(&bars.empty[s], ph);
         }
         if (!ok) break;
       }
@@ -310,14 +350,14 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
       const uint64_t dB = sdesc_sw128(smem_u32(smem + C::kABytes), 16, 1024);
       constexpr uint64_t kStageStep = (uint64_t)(C::kStageBytes >> 4);
       const uint32_t empty_own = smem_u32(&bars.empty[0]);
-      const uint32_t empty_peer = mapa_shared(empty_own, 1);
       const uint32_t accf_own = smem_u32(&bars.acc_full[0]);
-      const uint32_t accf_peer = mapa_shared(accf_own, 1);
       auto wait = [&](uint64_t* bar, uint32_t parity) {
         return __all_sync(0xffffffffu, mbar_wait(bar, parity, &abort_flag, tmo));
       };
       bool ok = true;
-      int k_it = 0, tc = 0;
+      int s = 0, tc = 0;
+      uint32_t ph = 0;  // of stage s's barrier
+      bool ready = false;  // stage s has landed
       for (int i = pair; ok && i < p.n_items; i += n_pairs, ++tc) {
         const uint32_t idesc = item_of(p, i).half >= 0 ? idesc_half : idesc_whole;
         const int acc = tc & 1;
@@ -327,28 +367,27 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
         }
         tc_fence_after();
         const uint32_t dcol = tbase + (uint32_t)(acc * BN);
-        for (int kb = 0; kb < p.n_kblocks; ++kb, ++k_it) {
-          const int s = k_it % kStages;
-          if (!wait(&bars.full[s], (uint32_t)(k_it / kStages) & 1u)) {
+        for (int kb = 0; kb < p.n_kblocks; ++kb) {
+          if (!__all_sync(0xffffffffu, ready) && !wait(&bars.full[s], ph)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint64_t a = dA + (uint64_t)s * kStageStep;
           const uint64_t b = dB + (uint64_t)s * kStageStep;
-#pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk)  // 32 bytes of K per MMA inside the swizzle atom
-            mma_ss_pair_warp(dcol, a + (uint64_t)(kk * 2), b + (uint64_t)(kk * 2), idesc,
-                             (kb > 0 || kk > 0) ? 1u : 0u);
+          const uint32_t done = empty_own + (uint32_t)(s * sizeof(uint64_t));
+          if (++s == kStages) {
+            s = 0;
+            ph ^= 1u;
+          }
+          ready = mbar_test_wait(&bars.full[s], ph);  // tested while these MMAs are issued
+          mma_ss_pair_warp_x4(dcol, a, b, idesc, kb > 0 ? 1u : 0u);
           // the stage is free in each CTA once these MMAs have read it
-          const uint32_t off = (uint32_t)(s * sizeof(uint64_t));
-          mma_commit_pair_warp(empty_own + off);
-          mma_commit_pair_warp(empty_peer + off);
+          mma_commit_both_warp(done);
         }
         if (!ok) break;
         const uint32_t off = (uint32_t)(acc * sizeof(uint64_t));
-        mma_commit_pair_warp(accf_own + off);
-        mma_commit_pair_warp(accf_peer + off);
+        mma_commit_both_warp(accf_own + off);
       }
       if (!ok && lane == 0) proj_timeout(p, &abort_flag);
     }
@@ -582,7 +621,7 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
   // again (bounded wait).  After a timeout the even CTA also waits for its
   // stage barriers, whose phases count both CTAs' copies, and for every MMA
   // it issued.
-  if (warp == 0 && lane == 0) {
+  if ((warp == 0 || warp == 2) && lane == 0) {
     const int zero = 0;
     for (int i = (issued > kStages ? issued - kStages : 0); i < issued; ++i) {
       mbar_wait(&bars.empty[i % kStages], (uint32_t)(i / kStages) & 1u, &zero, tmo);
