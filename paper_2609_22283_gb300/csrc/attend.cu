@@ -309,6 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
+  pdl_launch_dependents();
 
   // Work unit, head-major so the CTAs that share a head's K/V run together.
   // The first n_full units run unsplit (one CTA each, the full waves); the
@@ -399,6 +400,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       // Q and the first K tile are on their way while the CTA sets up the
       // rest: they used to follow the set-up, 600 cycles later.
       fence_proxy_async_smem();
+      pdl_wait();
       load_q();
       if (n_tiles > 0) {
         const int st = t_begin / p.nt_slot;
@@ -415,6 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     tmem_alloc(&tmem_base_sh, C::kTmemCols);
     tmem_relinquish();
   }
+  pdl_wait();  // everything above is this CTA's own; what follows reads and writes global memory
   if constexpr (sparse) if (warp == 2) {
     // Gather the caller's mask rows of the two query tiles into the kernel's
     // key tile order (slot list without hidden context slots), then take
@@ -1415,22 +1418,6 @@ cudaError_t configure_d(int dev) {
 }
 
 template <int D>
-void cluster_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int grid, int cluster,
-                    cudaStream_t s) {
-  *cfg = cudaLaunchConfig_t{};
-  cfg->gridDim = dim3((unsigned)grid, 1, 1);
-  cfg->blockDim = dim3(kThreads, 1, 1);
-  cfg->dynamicSmemBytes = AttnCfg<D>::kSmemBytes;
-  cfg->stream = s;
-  attr->id = cudaLaunchAttributeClusterDimension;
-  attr->val.clusterDim.x = (unsigned)cluster;
-  attr->val.clusterDim.y = 1;
-  attr->val.clusterDim.z = 1;
-  cfg->attrs = attr;
-  cfg->numAttrs = 1;
-}
-
-template <int D>
 cudaError_t launch_d(const AttnParams& p, int grid, cudaStream_t s) {
   using C = AttnCfg<D>;
   int dev = 0;
@@ -1439,21 +1426,14 @@ cudaError_t launch_d(const AttnParams& p, int grid, cudaStream_t s) {
   e = configure_d<D>(dev);
   if (e != cudaSuccess) return e;
   const bool token = p.masked && (p.own_mask != nullptr || p.hist_mask != nullptr);
-  if (p.cluster) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    cluster_config<D>(&cfg, &attr, grid, p.n_split, s);
-    return cudaLaunchKernelEx(&cfg, token      ? attend_kernel<D, true, true, true>
-                                    : p.masked ? attend_kernel<D, true, false, true>
-                                               : attend_kernel<D, false, false, true>, p);
-  }
-  if (token)
-    attend_kernel<D, true, true, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
-  else if (p.masked)
-    attend_kernel<D, true, false, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
-  else
-    attend_kernel<D, false, false, false><<<grid, kThreads, C::kSmemBytes, s>>>(p);
-  return cudaGetLastError();
+  LaunchConfig l(dim3((unsigned)grid), kThreads, C::kSmemBytes, s, p.cluster ? p.n_split : 0);
+  if (p.cluster)
+    return cudaLaunchKernelEx(&l.cfg, token      ? attend_kernel<D, true, true, true>
+                                      : p.masked ? attend_kernel<D, true, false, true>
+                                                 : attend_kernel<D, false, false, true>, p);
+  return cudaLaunchKernelEx(&l.cfg, token      ? attend_kernel<D, true, true, false>
+                                    : p.masked ? attend_kernel<D, true, false, false>
+                                               : attend_kernel<D, false, false, false>, p);
 }
 
 // Clusters of `size` CTAs (one CTA per SM) that can be resident at once on the
@@ -1469,11 +1449,9 @@ cudaError_t max_clusters_d(int size, int* out) {
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
   if (known[dev][size] == 0) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    cluster_config<D>(&cfg, &attr, size, size, nullptr);
+    LaunchConfig l(dim3((unsigned)size), kThreads, AttnCfg<D>::kSmemBytes, nullptr, size);
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, attend_kernel<D, false, false, true>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, attend_kernel<D, false, false, true>, &l.cfg);
     if (e != cudaSuccess) return e;
     known[dev][size] = n + 1;
   }

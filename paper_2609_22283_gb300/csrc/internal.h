@@ -118,6 +118,33 @@ constexpr size_t kStaticScratchBytes = (size_t)32 << 20;
 // first call on a device looks it up.  Defined in attend_noalloc.cu.
 cudaError_t static_split_scratch(int device, void** ptr);
 
+// A launch of `cluster` CTAs a cluster (0: none) with programmatic dependent
+// launch: every kernel of the library waits for the kernels before it
+// (pdl_wait) ahead of its first access to memory, so its launch and prologue
+// overlap their end.
+struct LaunchConfig {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  LaunchConfig(dim3 grid, int threads, size_t smem, cudaStream_t s, int cluster = 0) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 1;
+    if (cluster > 0) {
+      attr[1].id = cudaLaunchAttributeClusterDimension;
+      attr[1].val.clusterDim.x = (unsigned)cluster;
+      attr[1].val.clusterDim.y = 1;
+      attr[1].val.clusterDim.z = 1;
+      cfg.numAttrs = 2;
+    }
+    cfg.attrs = attr;
+  }
+  LaunchConfig(const LaunchConfig&) = delete;
+};
+
 // Launchers (defined in the .cu files).  They return the launch error.
 cudaError_t launch_attend(const AttnParams& p, int head_dim, int grid, cudaStream_t s);
 // Clusters of `size` attention CTAs that can be resident at once on the current device.

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace sva {
 namespace {
@@ -32,6 +33,8 @@ __global__ void __launch_bounds__(kWarps * 32) mask_scan_kernel(const __grid_con
   const int nt = (p.T + kTile - 1) / kTile;
   const uint32_t* mask = state == 0 ? p.own_mask : p.hist_mask;
   uint8_t* out = p.any + ((size_t)node * p.n_qt + qt) * p.row_bytes + (size_t)state * nt;
+  ptx::pdl_launch_dependents();
+  ptx::pdl_wait();
   if (state > p.n_ctx[node]) return;
   if (mask == nullptr) {
     for (int t = threadIdx.x; t < nt; t += kWarps * 32) out[t] = 1;
@@ -87,8 +90,8 @@ __global__ void __launch_bounds__(kWarps * 32) mask_scan_kernel(const __grid_con
 }  // namespace
 
 cudaError_t launch_mask_scan(const ScanParams& p, int n_nodes, int max_states, cudaStream_t s) {
-  mask_scan_kernel<<<dim3(max_states, p.n_qt, n_nodes), kWarps * 32, 0, s>>>(p);
-  return cudaGetLastError();
+  LaunchConfig l(dim3(max_states, p.n_qt, n_nodes), kWarps * 32, 0, s);
+  return cudaLaunchKernelEx(&l.cfg, mask_scan_kernel, p);
 }
 
 }  // namespace sva

@@ -36,6 +36,22 @@ __device__ __forceinline__ uint32_t elect_one_sync() {
   return pred;
 }
 
+// ---------------------------------------------------------------- launches
+//
+// Programmatic dependent launch: a kernel launched with the attribute may start
+// while the kernel before it in the stream still runs (once every block of that
+// one has called pdl_launch_dependents or exited), and calls pdl_wait before it
+// touches any memory that another kernel may write or read: pdl_wait returns
+// when every earlier kernel has completed and its writes are visible.
+
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

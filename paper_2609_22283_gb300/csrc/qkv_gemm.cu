@@ -265,6 +265,7 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
   const int pair = blockIdx.x >> 1;
   const int n_pairs = gridDim.x >> 1;
 
+  pdl_launch_dependents();
   if (threadIdx.x == 0) {
     prefetch_tmap(&p.tmap_x);
     prefetch_tmap(&p.tmap_w);
@@ -289,6 +290,7 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
   // both CTAs' barriers are initialised before either signals the other's
   cluster_sync();
   tc_fence_after();
+  pdl_wait();  // everything above is the pair's own; what follows reads and writes global memory
   const uint32_t tbase = tmem_base_sh;
   const uint64_t tmo = p.timeout_ns;
   int issued = 0;  // producer: K blocks whose copies were started
@@ -667,32 +669,14 @@ cudaError_t configure_bn(int dev) {
 }
 
 template <int BN>
-void pair_launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int grid,
-                        cudaStream_t s) {
-  *cfg = cudaLaunchConfig_t{};
-  cfg->gridDim = dim3((unsigned)grid, 1, 1);
-  cfg->blockDim = dim3(kProjThreads, 1, 1);
-  cfg->dynamicSmemBytes = ProjCfg<BN>::kSmemBytes;
-  cfg->stream = s;
-  attr->id = cudaLaunchAttributeClusterDimension;
-  attr->val.clusterDim.x = 2;
-  attr->val.clusterDim.y = 1;
-  attr->val.clusterDim.z = 1;
-  cfg->attrs = attr;
-  cfg->numAttrs = 1;
-}
-
-template <int BN>
 cudaError_t launch_bn(const ProjParams& p, int grid, cudaStream_t s) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   e = configure_bn<BN>(dev);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr;
-  pair_launch_config<BN>(&cfg, &attr, grid, s);
-  return cudaLaunchKernelEx(&cfg, qkv_project_kernel<BN>, p);
+  LaunchConfig l(dim3((unsigned)grid), kProjThreads, ProjCfg<BN>::kSmemBytes, s, 2);
+  return cudaLaunchKernelEx(&l.cfg, qkv_project_kernel<BN>, p);
 }
 
 // Clusters of two (one CTA per SM) that can be resident at once on the
@@ -709,11 +693,9 @@ cudaError_t max_pairs_bn(int* out) {
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
   if (pairs[dev] == 0) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
-    pair_launch_config<BN>(&cfg, &attr, 2, nullptr);
+    LaunchConfig l(dim3(2), kProjThreads, ProjCfg<BN>::kSmemBytes, nullptr, 2);
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, qkv_project_kernel<BN>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, qkv_project_kernel<BN>, &l.cfg);
     if (e != cudaSuccess) return e;
     if (n < 1) return cudaErrorInvalidConfiguration;
     pairs[dev] = n;

@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace sva {
 namespace {
@@ -88,6 +89,8 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
   __nv_bfloat16* cache = static_cast<__nv_bfloat16*>(p.cache);
   const int warps_per_block = blockDim.x >> 5;
   const int n_tok = p.n_nodes * p.T;
+  ptx::pdl_launch_dependents();
+  ptx::pdl_wait();
 
   for (int tok = blockIdx.x * warps_per_block + (threadIdx.x >> 5); tok < n_tok;
        tok += gridDim.x * warps_per_block) {
@@ -183,6 +186,8 @@ __global__ void __launch_bounds__(256, kVec <= 3 || !kQ ? 3 : 2)
   const size_t kv_stride = (size_t)p.H * p.Tpad * p.d;  // elements between K and V of a slot
   const int v0 = (warp % kWarps) * 32 + lane;
   const size_t in_tok = (size_t)tok * per_tok * 8;
+  ptx::pdl_launch_dependents();
+  ptx::pdl_wait();
   uint4 kv[kVec], qv[kQ ? kVec : 1], vv[kVec];
 #pragma unroll
   for (int j = 0; j < kVec; ++j) {
@@ -272,14 +277,12 @@ __global__ void __launch_bounds__(256, kVec <= 3 || !kQ ? 3 : 2)
 }
 
 template <int kWarps, int kVec>
-void launch_norm(const RopeParams& p, cudaStream_t s) {
+cudaError_t launch_norm(const RopeParams& p, cudaStream_t s) {
   const long long tokens = (long long)p.n_nodes * p.T;
   constexpr int per_block = 8 / kWarps;
-  const unsigned grid = (unsigned)((tokens + per_block - 1) / per_block);
-  if (p.q != nullptr)
-    rope_norm_kernel<kWarps, kVec, true><<<grid, 256, 0, s>>>(p);
-  else
-    rope_norm_kernel<kWarps, kVec, false><<<grid, 256, 0, s>>>(p);
+  LaunchConfig l(dim3((unsigned)((tokens + per_block - 1) / per_block)), 256, 0, s);
+  return p.q != nullptr ? cudaLaunchKernelEx(&l.cfg, rope_norm_kernel<kWarps, kVec, true>, p)
+                        : cudaLaunchKernelEx(&l.cfg, rope_norm_kernel<kWarps, kVec, false>, p);
 }
 
 }  // namespace
@@ -292,26 +295,17 @@ cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s) {
     // long as one token takes: 320 tokens of 12 x 128, 5.4 us at six vectors,
     // 4.0 at three), more where three would leave warps short of loads (40 x
     // 128: 38 us at three, 35 at five; 16 x 64: 13.5 at three, 12.6 at four).
-    if (per_tok <= 64)
-      launch_norm<1, 2>(p, s);
-    else if (per_tok <= 128)
-      launch_norm<1, 4>(p, s);
-    else if (per_tok <= 192)
-      launch_norm<2, 3>(p, s);
-    else if (per_tok <= 384)
-      launch_norm<4, 3>(p, s);
-    else if (per_tok <= 640)
-      launch_norm<4, 5>(p, s);
-    else if (per_tok <= 1280)
-      launch_norm<8, 5>(p, s);
-    else
-      launch_norm<8, 8>(p, s);
-  } else if (blocks <= 4LL * num_sms) {
-    rope_kv_kernel<true><<<p.grid_blocks, 256, 0, s>>>(p);
-  } else {
-    rope_kv_kernel<false><<<p.grid_blocks, 256, 0, s>>>(p);
+    if (per_tok <= 64) return launch_norm<1, 2>(p, s);
+    if (per_tok <= 128) return launch_norm<1, 4>(p, s);
+    if (per_tok <= 192) return launch_norm<2, 3>(p, s);
+    if (per_tok <= 384) return launch_norm<4, 3>(p, s);
+    if (per_tok <= 640) return launch_norm<4, 5>(p, s);
+    if (per_tok <= 1280) return launch_norm<8, 5>(p, s);
+    return launch_norm<8, 8>(p, s);
   }
-  return cudaGetLastError();
+  LaunchConfig l(dim3((unsigned)p.grid_blocks), 256, 0, s);
+  return blocks <= 4LL * num_sms ? cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<true>, p)
+                                 : cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<false>, p);
 }
 
 }  // namespace sva
