@@ -801,24 +801,35 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     auto state_of = [&](int tile) { return inv_nt ? (int)__umulhi((uint32_t)tile, inv_nt) : tile; };
     // Token-mask instance: this thread's bits of its row for a key tile, from
     // the own-chunk mask or from the history mask of the tile's key state (the
-    // caller's context index); all ones without such a mask.  Each is fetched
-    // a key tile ahead of its use: its L2 latency, on the path from S to P,
-    // cost about 0.1 us a tile.
-    auto token_bits = [&](int b, int tile, uint32_t (&ow)[NC]) {
+    // caller's context index); all ones without such a mask and for rows past
+    // T, which are never stored.  Each is fetched a key tile ahead of its use:
+    // its L2 latency, on the path from S to P, cost about 0.1 us a tile.  The
+    // rows' addresses are worked out once.
+    const uint32_t* own_row[NT];
+    const uint32_t* hist_row[NT];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) ow[c] = ~0u;
+    for (int x = 0; x < NT; ++x) {
+      const int u = (qt0 + (C::kOwnTile ? b_own : x)) * kTile + row;
+      const size_t qrow = (size_t)nd.q_index * p.T + u;
+      own_row[x] = kOwn && p.own_mask && u < p.T ? p.own_mask + qrow * p.own_words + half * 2 : nullptr;
+      hist_row[x] = kOwn && p.hist_mask && u < p.T
+                        ? p.hist_mask + qrow * p.hist_states * p.hist_words + half * 2
+                        : nullptr;
+    }
+    auto token_bits = [&](int x, int tile, uint32_t (&ow)[NC]) {
       const int st = state_of(tile);
-      const uint32_t* mask = st == 0 ? p.own_mask : p.hist_mask;
-      const int u = (qt0 + b) * kTile + row;
-      if (mask != nullptr && u < p.T) {  // rows past T are never stored
-        const size_t qrow = (size_t)nd.q_index * p.T + u;
-        const uint32_t* mrow =
-            mask + (st == 0 ? qrow * p.own_words
-                            : (qrow * p.hist_states + (nd.src[st] - 1)) * p.hist_words);
-        const int words = st == 0 ? p.own_words : p.hist_words;
-        const int wi = (tile - st * p.nt_slot) * 4 + half * 2;  // first key of this thread / 32
+      const int tt = tile - st * p.nt_slot;
+      const uint32_t* r = own_row[x];
+      int words = p.own_words;
+      if (st != 0) {
+        r = hist_row[x] ? hist_row[x] + (nd.src[st] - 1) * p.hist_words : nullptr;
+        words = p.hist_words;
+      }
+      words -= tt * 4 + half * 2;  // of this row from this thread's first on; < NC in the last tile only
 #pragma unroll
-        for (int c = 0; c < NC; ++c) ow[c] = wi + c < words ? __ldg(mrow + wi + c) : 0u;
+      for (int c = 0; c < NC; ++c) {
+        ow[c] = ~0u;
+        if (r) ow[c] = c < words ? __ldg(r + tt * 4 + c) : 0u;
       }
     };
     if constexpr (C::kOwnTile) {
@@ -867,7 +878,10 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           const int valid = own_fc ? min(valid_tile, frame_end[0] - t * kTile) : valid_tile;
           uint32_t w[NC];
 #pragma unroll
-          for (int c = 0; c < NC; ++c) w[c] = ow[c] & first_bits(valid - c * 32);
+          for (int c = 0; c < NC; ++c) w[c] = ow[c];
+          if (valid_tile < kTile || own_fc)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) w[c] &= first_bits(valid - c * 32);
           mask_tile(s, w, m_part, m[0], sl2);
         }
         const float m_tile = m_part * sl2;
@@ -937,7 +951,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 #pragma unroll
       for (int c = 0; c < NC; ++c) ow[c] = ~0u;
       if constexpr (kOwn)
-        if (my_tiles > 0) token_bits(b, kt, ow);
+        if (my_tiles > 0) token_bits(0, kt, ow);
       for (int i = 0; ok && i < my_tiles; ++i) {
         const int kt_next = sparse ? walk.next() : next_kt(kt);
         uint64_t* p_bar = &bars.p_full[b * 3 + bar];
@@ -957,7 +971,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           ok = row_max(i, s, cmax, ow);
           if (!ok) break;
           if constexpr (kOwn)
-            if (i + 1 < my_tiles) token_bits(b, kt_next, ow);
+            if (i + 1 < my_tiles) token_bits(0, kt_next, ow);
           const uint64_t negm = neg_max();
           uint64_t acc[4] = {0, 0, 0, 0};
           expo(s[0], negm, acc);
@@ -971,7 +985,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           add_sum(acc);
           o_has[0] = true;
         } else if constexpr (kOwn) {
-          if (i + 1 < my_tiles) token_bits(b, kt_next, ow);
+          if (i + 1 < my_tiles) token_bits(0, kt_next, ow);
         }
         mbar_arrive(p_bar);
         advance(kt_next);
@@ -1000,7 +1014,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         const uint32_t attends = sparse ? ((tmask[0][kt >> 5] >> (kt & 31)) & 1u) |
                                               (((tmask[1][kt >> 5] >> (kt & 31)) & 1u) << 1)
                                         : 3u;
-        const int t = kt % p.nt_slot;  // key tile inside its slot
+        const int t = sparse ? kt - state_of(kt) * p.nt_slot : kt % p.nt_slot;  // key tile inside its slot
         const int valid_tile = (t == p.nt_slot - 1) ? p.valid_last : kTile;
         const bool own_fc = frame_causal && kt < p.nt_slot;
 #pragma unroll
@@ -1041,7 +1055,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
             // row's latent frame are visible (tile 0, frame 0, always is)
             const int valid = own_fc ? min(valid_tile, frame_end[b] - t * kTile) : valid_tile;
             const int vrel = valid - half * 64;  // visible keys among this thread's 64
-            const uint32_t w[2] = {ow[b][0] & first_bits(vrel), ow[b][1] & first_bits(vrel - 32)};
+            uint32_t w[2] = {ow[b][0], ow[b][1]};
+            if (valid_tile < kTile || own_fc) {
+              w[0] &= first_bits(vrel);
+              w[1] &= first_bits(vrel - 32);
+            }
             mask_tile(s, w, m_part, m[b], sl2);
             if constexpr (kOwn)
               if (i + 1 < n_tiles) token_bits(b, kt_next, ow[b]);
