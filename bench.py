@@ -36,7 +36,7 @@ if ROOT not in sys.path:
 
 METRIC = "chunk-attention TFLOP/s (% of GB300 BF16 peak) and denoising nodes/s per layer"
 DEFAULT_WORKLOAD = "stress14b"
-KERNEL_SOURCES = ["paper_2609_22283_gb300/csrc/attend.cu", "paper_2609_22283_gb300/csrc/ptx.cuh",
+KERNEL_SOURCES = ["paper_2609_22283_gb300/csrc/attend.cuh", "paper_2609_22283_gb300/csrc/ptx.cuh",
                   "paper_2609_22283_gb300/csrc/internal.h"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "attend_dram_traffic.json")
 # Further full-geometry configurations timed beside the default one (attention

@@ -13,8 +13,8 @@
 // loads in flight.  A warp whose rows so far have set a bit in every tile
 // stops reading, so dense random masks cost a few rows per block.  One 4680-token node, 3 history
 // states, bits within 6 patch rows and columns (11 MB of masks): 7 us before
-// an attention launch that it shortens from 489 to 319 us (58% of the key tiles
-// of a query-tile pair keep a bit).
+// an attention launch that takes 394 us over every key tile and 262 us over the
+// 58% of them that keep a bit for the query-tile pair.
 #include <cuda_runtime.h>
 
 #include "internal.h"

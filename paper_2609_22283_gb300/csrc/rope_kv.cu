@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
 // (1150 MB) 204 -> 183 us; one node of 12 x 128 with Q 19.5 -> 19.4 us (a
 // device copy of its 43 MB takes 20.5 us in the same loop).
 template <int kWarps, int kVec, bool kQ>
-__global__ void __launch_bounds__(256, kVec <= 3 || !kQ ? 3 : 2)
+__global__ void __launch_bounds__(256, kVec <= 3 || (kVec <= 5 && !kQ) ? 3 : (kVec <= 5 || !kQ ? 2 : 1))
     rope_norm_kernel(const __grid_constant__ RopeParams p) {
   __shared__ float part[8][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
