@@ -106,3 +106,54 @@ def test_chains_of_calls(shape):
     assert torch.equal(a.x, ref) and torch.equal(b.x, ref)
     assert a.c.poll() == sva.OK and b.c.poll() == sva.OK
     a.c.close(), b.c.close()
+
+
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("shape", [0, 1])
+def test_fork_and_join(shape, captured):
+    """Two chains on two streams, joined by events into one tensor that the first chain reads next."""
+    a, b = Chain(seed=10, **SHAPES[shape]), Chain(seed=11, **SHAPES[shape])
+    fork = torch.empty_like(a.x)        # what b reads while a goes on to overwrite a.x
+
+    def step(main, side, wait=False):
+        with torch.cuda.stream(main):
+            a.steps(1)
+            fork.copy_(a.x)
+            side.wait_stream(main)
+            if wait:
+                torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            b.x.add_(fork)
+            b.steps(1)
+            if wait:
+                torch.cuda.synchronize()
+        with torch.cuda.stream(main):
+            a.steps(1)
+            main.wait_stream(side)      # our kernel next, straight after the join
+            a.c.qkv_project(b.x.view(1, a.T, a.N), a.w, a.b, a.q, a.k, a.v)
+            a.x.copy_(a.q)
+            if wait:
+                torch.cuda.synchronize()
+
+    def run(main, side, wait=False):
+        for _ in range(4):
+            step(main, side, wait)
+
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    run(main, side, wait=True)
+    ref = a.x.clone(), b.x.clone()
+    a.reset(), b.reset()
+    torch.cuda.synchronize()
+    if captured:
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=main):
+            run(main, side)
+        a.reset(), b.reset()
+        torch.cuda.synchronize()
+        g.replay()
+    else:
+        run(main, side)
+    torch.cuda.synchronize()
+    assert torch.equal(a.x, ref[0]) and torch.equal(b.x, ref[1])
+    a.c.close(), b.c.close()
