@@ -352,10 +352,11 @@ sva_status sva_cache_set_workspace(sva_cache* c, void* dev_buf, size_t bytes);
  * workspace of sva_cache_set_workspace.  This entry point takes the same
  * arguments, runs the same checks and chooses the same key-range split plan
  * as sva_attend_nodes with a workspace attached, so its results are bitwise
- * the same, but it keeps its key-range partials and arrival counters in a
- * scratch array that the library declares in device memory itself (32 MiB,
- * held by every GPU that loads the library until the process exits).  It
- * allocates nothing and calls no allocating routine.  Launches whose split
+ * the same, but where that plan uses the workspace it keeps its key-range
+ * partials and arrival counters in a scratch array that the library declares
+ * in device memory itself (32 MiB, held by every GPU that loads the library
+ * until the process exits).  It allocates nothing and calls no allocating
+ * routine.  Launches whose split
  * plan needs more than 32 MiB of scratch (counters plus 133 KB per split
  * item at head_dim 128) are rejected with SVA_ERR_CAPACITY and launch
  * nothing; launches that need no split use no scratch and are never
