@@ -55,15 +55,18 @@ __global__ void __launch_bounds__(kWarps * 32) mask_scan_kernel(const __grid_con
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const int w = base + j * 32 + lane;
-        v[j] = w < words ? __ldg(row + w) : ~0u;
-        v2[j] = w < words ? __ldg(row2 + w) : ~0u;
+        v[j] = w < words ? __ldg(row + w) : 0u;
+        v2[j] = w < words ? __ldg(row2 + w) : 0u;
       }
-      // every tile (four words, four neighbouring lanes) has a bit by now?
+      // every tile (four words, four neighbouring lanes) has a bit by now, or
+      // lies past the row's end?  The words that the last tile lacks must not
+      // stand in for the ones it has.
       bool all = true;
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         acc[j] |= v[j] | v2[j];
-        const uint32_t has = __ballot_sync(0xffffffffu, acc[j] != 0u);
+        const bool past = base + j * 32 + (lane & ~3) >= words;
+        const uint32_t has = __ballot_sync(0xffffffffu, past || acc[j] != 0u);
         const uint32_t pair = has | (has >> 1);
         all = all && ((pair | (pair >> 2)) & 0x11111111u) == 0x11111111u;
       }
@@ -79,8 +82,7 @@ __global__ void __launch_bounds__(kWarps * 32) mask_scan_kernel(const __grid_con
 #pragma unroll
       for (int w = 0; w < kWarps; ++w)
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (base + (int)threadIdx.x * 4 + k < words) any |= seen[w][threadIdx.x * 4 + k];
+        for (int k = 0; k < 4; ++k) any |= seen[w][threadIdx.x * 4 + k];
       out[t] = any != 0u;
     }
     __syncthreads();

@@ -156,3 +156,53 @@ def test_scan_of_empty_tiles(form, d):
     assert ((a - b).abs() <= 2.0 ** -8 * (a.abs() + b.abs()) + 2 * 2.0 ** -8 * v_max).all()
     assert float((a - b).norm() / b.norm()) <= 5e-3
     cache.close()
+
+
+# Masks whose rows all see every full key tile, so that a warp of the scan has a bit in each of them
+# after its first rows, and whose ragged last tile only the last rows of every query tile see: it may
+# not be given up before all rows are read.  With `rare` a full tile is seen by one row in 256 as
+# well.  T leaves 1 to 4 words in the last tile, or has more words than one pass over a row takes
+# (256).  The keys of those tiles are large, so that a row which lost them is off by far more than
+# the bound.
+@pytest.mark.parametrize("rare", [False, True])
+@pytest.mark.parametrize("which", ["own", "history"])
+@pytest.mark.parametrize("T,H,W", [(2580, 12, 4), (2610, 12, 4), (2500, 12, 4), (2680, 12, 4), (2560, 12, 4),
+                                   (8220, 4, 1)])
+def test_scan_reads_every_row(T, H, W, which, rare):
+    d, nt, words = 64, -(-T // 128), -(-T // 32)
+    assert H * -(-nt // 2) * (W + 1) * nt >= 12000    # the size from which masks are scanned
+    cache = sva.Cache(sva.make_geometry(H, d, 1, 1, T, num_slots=W + 1, pairs=rope_pairs_for(d), max_frames=W + 4))
+    gen = torch.Generator(device="cuda").manual_seed(T)
+    draw = lambda: torch.randn((1, T, H, d), generator=gen, device="cuda")  # noqa: E731
+    last, few = (nt - 1) * 128, 3 * 128      # first keys of the last tile and of the rarely seen one
+    slots = []
+    for b in range(W + 1, 0, -1):
+        k = draw()
+        k[0, last:] *= 40.0
+        k[0, few:few + 128] *= 40.0
+        s = cache.bind(0, b, 0)
+        cache.rope_kv_write([dict(seq=0, chunk=b, level=0, own_slot=s)], k.bfloat16(), draw().bfloat16())
+        slots.append(s)
+    nodes = sva.make_nodes([dict(seq=0, chunk=W + 1, level=0, own_slot=slots[0], ctx=slots[1:])])
+    q = draw().bfloat16()
+    m = torch.full((1, T, words), -1, dtype=torch.int32, device="cuda")
+    u = torch.arange(T, device="cuda")
+    m[0, :, last // 32:][(u % 128 < 110) & (u < T - 5)] = 0
+    if rare:
+        m[0, :, few // 32:few // 32 + 4][u % 256 != 255] = 0
+    own = m if which == "own" else None
+    hist = m[:, :, None].repeat(1, 1, W, 1) if which == "history" else None
+    got = []
+    for ws in (False, True):
+        if ws:
+            cache.set_workspace(torch.empty(cache.workspace_bytes(), dtype=torch.uint8, device="cuda"))
+        out, lse = torch.empty_like(q), torch.empty((1, H, T), device="cuda")
+        cache.attend_nodes_masked(nodes, q, out, lse, own_mask=own, hist_mask=hist)
+        assert cache.poll() == sva.OK
+        got.append((out.double(), lse.double()))
+    (a, la), (b, lb) = got
+    # the same logits in either path; the fp32 sums over the keys in another order
+    assert ((la - lb).abs() <= 1e-3 + 2.0 ** -20 * la.abs()).all()
+    v_max = float(cache.slot_pool()[:, 1].abs().max())
+    assert ((a - b).abs() <= 2.0 ** -8 * (a.abs() + b.abs()) + 2 * 2.0 ** -8 * v_max).all()
+    cache.close()
