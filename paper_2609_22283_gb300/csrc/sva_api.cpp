@@ -874,11 +874,14 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
                     "workspace for launches this large)",
                     split_units, split0, need, sva::kStaticScratchBytes);
     }
+    // Looked up also where this launch needs no scratch: the first look-up on
+    // a device loads the array, which may not happen in a later call that is
+    // being captured.
+    void* addr = nullptr;
+    cudaError_t e = sva::static_split_scratch(c->device, &addr);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(split scratch)");
     if (use_ws) {
       counter_bytes = round_up((size_t)(units - n_full) * 4, 256);
-      void* addr = nullptr;
-      cudaError_t e = sva::static_split_scratch(c->device, &addr);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(split scratch)");
       split_base = static_cast<char*>(addr);
     }
   }

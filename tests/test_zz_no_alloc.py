@@ -14,6 +14,8 @@ partial last wave split).  This file runs last so that a failure here cannot
 hide the results of the other tests, and it depends on no state they leave
 behind."""
 import ctypes
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -23,6 +25,7 @@ from paper_2609_22283_gb300 import inputs as I
 from paper_2609_22283_gb300 import sva
 from paper_2609_22283_gb300.pipeline import Step
 from tests import _parity as P
+from tests.conftest import ROOT
 
 pytestmark = pytest.mark.gpu
 
@@ -161,3 +164,48 @@ def test_plan_mirror_on_152_sms():
     assert units == 228 and _plan(units, 4 * w.tiles, 152, 4 * 152) == (152, 2)
     n_split, need = _scratch(w, 152)
     assert n_split == 2 and need == 512 + 76 * 2 * 256 * (128 + 2) * 4   # counters + partials
+
+
+_CAPTURE = """
+import torch
+from paper_2609_22283_gb300 import inputs as I
+from paper_2609_22283_gb300 import sva
+from paper_2609_22283_gb300.pipeline import Step
+from tests.test_zz_no_alloc import SPLIT4, _noalloc
+
+def ready(w):
+    step, inp = Step(w, workspace=False), I.generate(w)
+    step.prefill(inp)
+    q, k, v = step.device_inputs(inp)
+    nodes, _ = step.node_table()
+    step.cache.rope_kv_write(nodes, k, v, q, check=False)
+    return step, nodes, q, *step.outputs()
+
+small, large = ready(SPLIT4), ready(I.WORKLOADS["clean1"])
+torch.cuda.synchronize()
+assert _noalloc(*small) == sva.OK, sva.last_error()      # the first call on the device
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):
+    free = torch.cuda.mem_get_info()[0]
+    st = _noalloc(*large)
+    taken = free - torch.cuda.mem_get_info()[0]
+assert st == sva.OK, sva.last_error()
+assert taken == 0, f"the captured call took {taken} bytes of device memory"
+g.replay()
+assert large[0].cache.poll() == sva.OK
+got = large[3].clone(), large[4].clone()
+assert _noalloc(*large) == sva.OK
+torch.cuda.synchronize()
+assert torch.equal(got[0], large[3]) and torch.equal(got[1], large[4])
+print("captured")
+"""
+
+
+def test_first_call_readies_a_capture():
+    """The first call on a device, small enough to use no scratch, looks the
+    scratch up all the same, so that a later call that does use it can be
+    captured and takes no device memory.  In a process of its own: the look-up
+    is made once per process."""
+    r = subprocess.run([sys.executable, "-c", _CAPTURE], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "captured" in r.stdout, r.stderr[-2000:]
