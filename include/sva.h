@@ -356,19 +356,24 @@ sva_status sva_cache_set_workspace(sva_cache* c, void* dev_buf, size_t bytes);
  * partials and arrival counters in a scratch array that the library declares
  * in device memory itself (32 MiB, held by every GPU that loads the library
  * until the process exits).  It allocates nothing and calls no allocating
- * routine.  Launches whose split
- * plan needs more than 32 MiB of scratch (counters plus 133 KB per split
- * item at head_dim 128) are rejected with SVA_ERR_CAPACITY and launch
- * nothing; launches that need no split use no scratch and are never
- * rejected for size.
+ * routine.
+ * Its size limit is stated for the wave-filling split of a launch, whether or
+ * not the plan makes that split: s ranges per work unit, for the smallest s in
+ * 1..4 that minimises ceil(units * s / SMs) / s with at least 4 key tiles in a
+ * range, of every unit or, where that is no slower, of the units past the last
+ * full wave of one unit per SM.  Launches whose wave-filling split needs more
+ * than 32 MiB of scratch (counters plus 133 KB per range at head_dim 128) are
+ * rejected with SVA_ERR_CAPACITY and launch nothing, also where the plan would
+ * merge inside clusters or run unsplit and use no scratch; launches whose
+ * wave-filling split is s = 1 are never rejected for size.
  * Each call clears the array's counters on `s` before its kernel; the
  * partials left by one call are overwritten by the next.  All calls on a
  * device share the one array, so calls whose kernels can overlap on the
  * GPU (different streams without ordering between them) race and must not
  * be issued.  The first call on a device looks up the array's device
- * address (cudaGetSymbolAddress); make that first call before any stream
- * capture.  The paper has no counterpart of this entry point.
- * Errors: as sva_attend_nodes, plus CAPACITY for a plan that does not fit. */
+ * address (cudaGetSymbolAddress), whatever its size; make that first call
+ * before any stream capture.  The paper has no counterpart of this entry point.
+ * Errors: as sva_attend_nodes, plus CAPACITY beyond that limit. */
 sva_status sva_attend_nodes_noalloc(sva_cache* c, const sva_node* nodes, int32_t n_nodes,
                                     const void* q, void* out, float* lse, float scale,
                                     sva_stream s);

@@ -807,8 +807,8 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
                     i, (long long)p.nodes[i].n_kv * p.nt_slot, 32 * sva::kMaskWords);
 
   // The split plan.  The static scratch takes the plan a full caller
-  // workspace would get, so both entry points compute the same result, and
-  // refuses a plan whose partials do not fit the array.
+  // workspace would get, so both entry points compute the same result, within
+  // a limit of its own (below).
   int min_tiles = 1 << 30;
   for (int i = 0; i < n_nodes; ++i)
     min_tiles = std::min(min_tiles, key_tiles_walked(c, p.nodes[i], p.nt_slot));
@@ -859,7 +859,9 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
   if (scratch == Scratch::kStatic) {
     split_base = nullptr;
     // The limit of this entry point is stated for the wave-filling split, also
-    // where the launch turns out to need less scratch or none.
+    // where the plan turns out to need less scratch or none: callers have sized
+    // their launches by it since before plans counted the cost of a merge.  A
+    // plan that uses the workspace is that split, so it always fits.
     long long full0 = 0;
     int split0 = 1;
     plan_split(c, units, min_tiles, cap, &full0, &split0);
@@ -869,9 +871,9 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
                           (size_t)split_units * split0 * ws_item_bytes(c);
       if (need > sva::kStaticScratchBytes)
         return fail(SVA_ERR_CAPACITY,
-                    "this launch splits %lld work units %d ways and needs %zu bytes of scratch; the "
-                    "library's static scratch holds %zu bytes (use sva_attend_nodes with a "
-                    "workspace for launches this large)",
+                    "the wave-filling split of this launch, %lld work units %d ways, needs %zu bytes "
+                    "of scratch; the library's static scratch holds %zu bytes (use sva_attend_nodes "
+                    "with a workspace for launches this large)",
                     split_units, split0, need, sva::kStaticScratchBytes);
     }
     // Looked up also where this launch needs no scratch: the first look-up on

@@ -7,10 +7,11 @@ Through the C ABI, on two calls in a row, its output must match what
 sva_attend_nodes with a workspace computes on the same inputs, within the
 tolerances of the other parity tests (and, since both take the same split
 plan, bit for bit); on clean1 it is also checked against the oracle.  A
-launch whose split plan needs more scratch than the array holds must be
-refused without launching anything.  The expected plans are worked out here
-from the device's SM count with the planner's rule (full waves unsplit, the
-partial last wave split).  This file runs last so that a failure here cannot
+launch whose wave-filling split needs more scratch than the array holds must
+be refused without launching anything.  That split, by which the limit is
+stated, is worked out here from the device's SM count (full waves unsplit, the
+partial last wave split); the plan that a launch takes also counts what a
+merge costs and may merge inside clusters or not split at all.  This file runs last so that a failure here cannot
 hide the results of the other tests, and it depends on no state they leave
 behind."""
 import ctypes
@@ -35,14 +36,21 @@ STATIC_SCRATCH = 32 << 20
 MAX_SPLIT = 4
 
 # 1 node, 2 heads x 128, T = 240, clean history of 7 chunks: 2 work units of
-# 16 key tiles each, which the split plan divides 4 ways (about 1 MB of scratch).
+# 16 key tiles each, whose wave-filling split is 4 ways (about 1 MB of scratch)
+# and which are merged inside clusters.
 SPLIT4 = I.Workload(name="split4", seed=9, F=1, Hp=8, Wp=30, H=2, d=128, K=4, W=7,
                     policy="clean", nodes=((0, 9, 4),),
                     prefilled=tuple((0, c, 0) for c in range(2, 9)))
 
+# 8 sequences of the same, 20 heads: 160 work units, one wave of 152 unsplit and
+# 8 split 4 ways, merged through the scratch.
+MERGE4 = I.Workload(name="merge4", seed=10, F=1, Hp=8, Wp=30, H=20, d=128, K=4, W=7,
+                    policy="clean", nodes=tuple((s, 9, 4) for s in range(8)),
+                    prefilled=tuple((s, c, 0) for s in range(8) for c in range(2, 9)))
+
 
 def _plan(units, min_tiles, sms, cap):
-    """(n_full, n_split) as the library plans a launch: the number of splits
+    """(n_full, n_split) of the wave-filling split: the number of splits
     minimising waves per split, the full waves unsplit when that is no worse."""
     def choose(u):
         best, best_s = float(-(-u // sms)), 1
@@ -65,7 +73,7 @@ def _plan(units, min_tiles, sms, cap):
 
 
 def _scratch(w, sms):
-    """(n_split, bytes of static scratch) of a dense launch of workload w."""
+    """(n_split, bytes of scratch) of the wave-filling split of a dense launch of workload w."""
     nt = w.tiles
     units = w.H * w.n_nodes * -(-nt // 2)
     min_tiles = min((1 + max(0, min(w.W, b - 1))) * nt for (_, b, _) in w.nodes)
@@ -88,12 +96,12 @@ def _noalloc(step, nodes, q, out, lse):
         step.scale, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
 
 
-@pytest.mark.parametrize("name", ["split4", "tiny", "clean1"])
+@pytest.mark.parametrize("name", ["split4", "merge4", "tiny", "clean1"])
 def test_noalloc_matches_attend_nodes_twice(name):
-    w = SPLIT4 if name == "split4" else I.WORKLOADS[name]
+    w = {"split4": SPLIT4, "merge4": MERGE4}.get(name) or I.WORKLOADS[name]
     n_split, need = _scratch(w, _sms())
-    if name in ("split4", "clean1"):
-        assert n_split > 1 and 0 < need <= STATIC_SCRATCH, (n_split, need)   # the split path
+    if name != "tiny":
+        assert n_split > 1 and 0 < need <= STATIC_SCRATCH, (n_split, need)
     inp = I.generate(w)
     step = Step(w, workspace=True)
     step.prefill(inp)
@@ -129,8 +137,8 @@ def test_noalloc_matches_attend_nodes_twice(name):
 
 def test_noalloc_refuses_plan_beyond_its_scratch():
     # One node of 240 tokens (one work unit per head, 16 key tiles) over 7
-    # clean history chunks; the head count is the smallest whose split plan
-    # on this GPU needs more than the static scratch.
+    # clean history chunks; the head count is the smallest whose wave-filling
+    # split on this GPU needs more than the static scratch.
     sms = _sms()
     w = None
     for H in range(1, 129):
@@ -153,16 +161,26 @@ def test_noalloc_refuses_plan_beyond_its_scratch():
     torch.cuda.synchronize()
     assert bool((out == 7.0).all())                # nothing was launched
     assert step.cache.poll() == sva.OK
+    # The limit is that of the wave-filling split: the plan itself does not
+    # split this launch, which leaves a workspace as it was.
+    ws = torch.empty(step.cache.workspace_bytes(), dtype=torch.uint8, device="cuda")
+    step.cache.set_workspace(ws)
+    ws.fill_(0xA5)
+    step.cache.attend_nodes(nodes, q, out, None, step.scale)
+    assert step.cache.poll() == sva.OK
+    assert bool((ws == 0xA5).all()) and not bool((out == 7.0).all())
     step.close()
 
 
 def test_plan_mirror_on_152_sms():
-    """The expected plans used above, on the GB300's 152 SMs: clean1 runs 152
-    units whole and splits the other 76 two ways (about 20 MB of scratch)."""
+    """The wave-filling splits used above, on the GB300's 152 SMs: clean1 has 152
+    units whole and the other 76 two ways (about 20 MB of scratch), merge4 152
+    and 8 four ways."""
     w = I.WORKLOADS["clean1"]
     units = w.H * -(-w.tiles // 2)
     assert units == 228 and _plan(units, 4 * w.tiles, 152, 4 * 152) == (152, 2)
     n_split, need = _scratch(w, 152)
+    assert _plan(160, 16, 152, 4 * 152) == (152, 4)
     assert n_split == 2 and need == 512 + 76 * 2 * 256 * (128 + 2) * 4   # counters + partials
 
 
