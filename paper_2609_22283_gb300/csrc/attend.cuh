@@ -1190,7 +1190,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       // up its columns in order of the key ranges.  So the merge is spread
       // over the unit's CTAs (131 KB out and in per CTA at D = 128, whatever
       // ns), needs no workspace, and costs two cluster barriers instead of
-      // stores to L2, a fence, an atomic and the last CTA's reads.
+      // stores to L2, a fence, an atomic and the last CTA's reads.  A range
+      // that timed out sends l = -1 in place of its rows, and no owner writes
+      // those: what its partial would have been is not in shared memory.
       constexpr int kGroups8 = D / 8;
       const int per = (kGroups8 + ns - 1) / ns;  // column groups per owner
       const uint32_t data = smem_u32(smem);
@@ -1235,6 +1237,16 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
               st_cluster_f32(dst + 1024, l_row[x]);
             }
         }
+      } else {
+#pragma unroll
+        for (int x = 0; x < NT; ++x)
+          if (half == 0)
+            for (int k = 0; k < ns; ++k) {
+              const int r = (C::kOwnTile ? b_own : x) * 128 + row;
+              const uint32_t dst = mapa_shared(ml + (uint32_t)(split * 2048 + r * 4), (uint32_t)k);
+              st_cluster_f32(dst, -INFINITY);
+              st_cluster_f32(dst + 1024, -1.0f);
+            }
       }
       __syncwarp();
       cluster_sync();  // every partial has arrived; nothing is read from another CTA after this
@@ -1246,19 +1258,22 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         const float M_sub = (M == -INFINITY) ? 0.0f : M;  // every range empty: O = 0
         float w[kMaxClusterSplit];
         float L = 0.0f;
+        bool whole = true;  // every range has sent this row
 #pragma unroll
         for (int k = 0; k < kMaxClusterSplit; ++k) {
           w[k] = 0.0f;
           if (k < ns) {
             const uint32_t at = ml + (uint32_t)(k * 2048 + r * 4);
-            w[k] = ld_shared_f32(at + 1024) * ex2(ld_shared_f32(at) - M_sub);
+            const float l_k = ld_shared_f32(at + 1024);
+            whole = whole && !(l_k < 0.0f);
+            w[k] = l_k * ex2(ld_shared_f32(at) - M_sub);
             L += w[k];
           }
         }
         const float inv_L = L > 0.0f ? 1.0f / L : 0.0f;
         uint4* orow4 = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) +
                                                 (((size_t)nd.q_index * p.T + token) * p.H + h) * D);
-        for (int g = 0; g < per && split * per + g < kGroups8; ++g) {
+        for (int g = 0; whole && g < per && split * per + g < kGroups8; ++g) {
           float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int k = 0; k < kMaxClusterSplit; ++k) {
@@ -1275,7 +1290,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           orow4[split * per + g] = make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]),
                                               pack_bf16(a[4], a[5]), pack_bf16(a[6], a[7]));
         }
-        if (p.lse != nullptr && split == 0)
+        if (whole && p.lse != nullptr && split == 0)
           p.lse[((size_t)nd.q_index * p.H + h) * p.T + token] = (M + __log2f(L)) * 0.69314718055994531f;
       }
     } else if (ns == 1) {
