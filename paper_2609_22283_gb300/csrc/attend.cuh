@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         ow[c] = ~0u;
-        if (r) ow[c] = c < words ? __ldg(r + tt * 4 + c) : 0u;
+        if (r) ow[c] = ld_global_u32_if(r + tt * 4 + c, c < words, 0u);
       }
     };
     if constexpr (C::kOwnTile) {

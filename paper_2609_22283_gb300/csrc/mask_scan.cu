@@ -55,8 +55,8 @@ __global__ void __launch_bounds__(kWarps * 32) mask_scan_kernel(const __grid_con
 #pragma unroll
       for (int j = 0; j < kGroup; ++j) {
         const int w = base + j * 32 + lane;
-        v[j] = w < words ? __ldg(row + w) : 0u;
-        v2[j] = w < words ? __ldg(row2 + w) : 0u;
+        v[j] = ptx::ld_global_u32_if(row + w, w < words, 0u);
+        v2[j] = ptx::ld_global_u32_if(row2 + w, w < words, 0u);
       }
       // every tile (four words, four neighbouring lanes) has a bit by now, or
       // lies past the row's end?  The words that the last tile lacks must not

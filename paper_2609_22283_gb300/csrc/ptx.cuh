@@ -52,6 +52,35 @@ __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Loads of what a caller passes: an earlier kernel may still be writing it
+// while this one is resident ahead of its pdl_wait.  The read-only path (__ldg,
+// ld.global.nc) is defined only for memory that nothing writes as long as the
+// kernel runs, so it is kept for the rotation tables; these are ordinary loads,
+// which stay behind pdl_wait (both are volatile).
+
+__device__ __forceinline__ float4 ld_global_f4(const void* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+
+// One word, or `other` without a load where `load` is false.
+__device__ __forceinline__ uint32_t ld_global_u32_if(const uint32_t* p, bool load, uint32_t other) {
+  uint32_t v;
+  asm volatile(
+      "{\n"
+      " .reg .pred q;\n"
+      " setp.ne.u32 q, %2, 0;\n"
+      " mov.b32 %0, %3;\n"
+      " @q ld.global.u32 %0, [%1];\n"
+      "}\n"
+      : "=&r"(v)
+      : "l"(p), "r"((uint32_t)load), "r"(other));
+  return v;
+}
+
 // ---------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

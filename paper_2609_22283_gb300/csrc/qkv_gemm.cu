@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
           const float4* b4 = reinterpret_cast<const float4*>(p.bias + col + c * 32);
 #pragma unroll
           for (int v = 0; v < 8; ++v) {
-            const float4 x = __ldg(b4 + v);
+            const float4 x = ld_global_f4(b4 + v);
             bv[4 * v] = x.x; bv[4 * v + 1] = x.y; bv[4 * v + 2] = x.z; bv[4 * v + 3] = x.w;
           }
         } else {
@@ -536,11 +536,11 @@ __global__ void __launch_bounds__(kProjThreads, 1) qkv_project_kernel(const __gr
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
             const int pi = ci * 16 + e;
-            const float2* a =
+            const float2* tab =
                 pi < rp.P0 ? pt + pi
                            : (pi < rp.P0 + rp.P1 ? rp.tab_h + (size_t)(pi - rp.P0) * rp.Hp + hh
                                                  : rp.tab_w + (size_t)(pi - rp.P0 - rp.P1) * rp.Wp + ww);
-            cs[e] = __ldg(a);
+            cs[e] = __ldg(tab);
           }
         };
         float2 cs_next[16];

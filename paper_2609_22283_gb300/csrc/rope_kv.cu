@@ -23,7 +23,7 @@ namespace {
 
 __device__ __forceinline__ uint4 ld_stream(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
@@ -258,8 +258,8 @@ __global__ void __launch_bounds__(256, kVec <= 3 || (kVec <= 5 && !kQ) ? 3 : (kV
   const float rq = __frsqrt_rn(__fmaf_rn(sq, inv_n, p.norm_eps));
   // x * gamma / rms of one vector, rotated
   auto norm_rotate = [&](uint4 x, const float* gamma, int v, float r) {
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gamma + (size_t)v * 8));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gamma + (size_t)v * 8) + 1);
+    const float4 g0 = ptx::ld_global_f4(gamma + (size_t)v * 8);
+    const float4 g1 = ptx::ld_global_f4(gamma + (size_t)v * 8 + 4);
     return make_uint4(norm_rotate_pair(x.x, g0.x * r, g0.y * r, cs[0].x, cs[0].y),
                       norm_rotate_pair(x.y, g0.z * r, g0.w * r, cs[1].x, cs[1].y),
                       norm_rotate_pair(x.z, g1.x * r, g1.y * r, cs[2].x, cs[2].y),
