@@ -64,6 +64,27 @@ __device__ __forceinline__ uint32_t rotate_pair(uint32_t xy, float c, float s) {
   return *reinterpret_cast<uint32_t*>(&r);
 }
 
+// The gammas of a vector of eight.  They come by ordinary loads, which the
+// compiler keeps behind the stores in front of them, so a vector's
+// gammas are fetched ahead of the stores of the vector before it.  (Fetched at
+// their use the write with Q took 3 to 10% longer at every size; all fetched
+// ahead of the first store they spill, up to 40% longer.)
+struct Gamma8 {
+  float4 lo, hi;
+};
+__device__ __forceinline__ Gamma8 gamma_at(const float* gamma, int v) {
+  return {ptx::ld_global_f4(gamma + (size_t)v * 8), ptx::ld_global_f4(gamma + (size_t)v * 8 + 4)};
+}
+
+// x * gamma * r of one vector, rotated
+__device__ __forceinline__ uint4 norm_rotate(uint4 x, const Gamma8& g, float r,
+                                             const float2 (&cs)[4]) {
+  return make_uint4(norm_rotate_pair(x.x, g.lo.x * r, g.lo.y * r, cs[0].x, cs[0].y),
+                    norm_rotate_pair(x.y, g.lo.z * r, g.lo.w * r, cs[1].x, cs[1].y),
+                    norm_rotate_pair(x.z, g.hi.x * r, g.hi.y * r, cs[2].x, cs[2].y),
+                    norm_rotate_pair(x.w, g.hi.z * r, g.hi.w * r, cs[3].x, cs[3].y));
+}
+
 // One warp per (node, token).  A token's H*d values are contiguous in the
 // token-major inputs, so the warp walks them as 16-byte vectors; lane l always
 // holds vector l mod (d/8) of a head row, i.e. the same four pairs for every
@@ -253,25 +274,26 @@ __global__ void __launch_bounds__(256, kVec <= 3 || (kVec <= 5 && !kQ) ? 3 : (kV
     const int v = v0 + j * 32 * kWarps;
     if (v < per_tok) *reinterpret_cast<uint4*>(cache_at(v) + kv_stride) = vv[j];
   }
+  Gamma8 next{};  // the gammas of the next vector to be stored
+  if (v0 < per_tok) next = gamma_at(p.gamma_k, v0);
   const float inv_n = 1.0f / (float)(per_tok * 8);
   const float rk = __frsqrt_rn(__fmaf_rn(sk, inv_n, p.norm_eps));
   const float rq = __frsqrt_rn(__fmaf_rn(sq, inv_n, p.norm_eps));
-  // x * gamma / rms of one vector, rotated
-  auto norm_rotate = [&](uint4 x, const float* gamma, int v, float r) {
-    const float4 g0 = ptx::ld_global_f4(gamma + (size_t)v * 8);
-    const float4 g1 = ptx::ld_global_f4(gamma + (size_t)v * 8 + 4);
-    return make_uint4(norm_rotate_pair(x.x, g0.x * r, g0.y * r, cs[0].x, cs[0].y),
-                      norm_rotate_pair(x.y, g0.z * r, g0.w * r, cs[1].x, cs[1].y),
-                      norm_rotate_pair(x.z, g1.x * r, g1.y * r, cs[2].x, cs[2].y),
-                      norm_rotate_pair(x.w, g1.z * r, g1.w * r, cs[3].x, cs[3].y));
-  };
 #pragma unroll
   for (int j = 0; j < kVec; ++j) {
     const int v = v0 + j * 32 * kWarps;
     if (v < per_tok) {
-      *reinterpret_cast<uint4*>(cache_at(v)) = norm_rotate(kv[j], p.gamma_k, v, rk);
-      if constexpr (kQ)
-        *reinterpret_cast<uint4*>(qio + in_tok + (size_t)v * 8) = norm_rotate(qv[j], p.gamma_q, v, rq);
+      const bool more = j + 1 < kVec && v + 32 * kWarps < per_tok;
+      Gamma8 g = next;  // of this vector's K, then of its Q
+      if constexpr (kQ) next = gamma_at(p.gamma_q, v);
+      const uint4 k = norm_rotate(kv[j], g, rk, cs);
+      if (!kQ && more) next = gamma_at(p.gamma_k, v + 32 * kWarps);
+      *reinterpret_cast<uint4*>(cache_at(v)) = k;
+      if constexpr (kQ) {
+        g = next;
+        if (more) next = gamma_at(p.gamma_k, v + 32 * kWarps);
+        *reinterpret_cast<uint4*>(qio + in_tok + (size_t)v * 8) = norm_rotate(qv[j], g, rq, cs);
+      }
     }
   }
 }
