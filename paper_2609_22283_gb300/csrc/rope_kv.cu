@@ -65,8 +65,8 @@ __device__ __forceinline__ uint32_t rotate_pair(uint32_t xy, float c, float s) {
 }
 
 // The gammas of a vector of eight.  They come by ordinary loads, which the
-// compiler keeps behind the stores in front of them, so a vector's
-// gammas are fetched ahead of the stores of the vector before it.  (Fetched at
+// compiler keeps behind the stores in front of them, so both kernels fetch a
+// vector's gammas ahead of the stores of the vector before it.  (Fetched at
 // their use the write with Q took 3 to 10% longer at every size; all fetched
 // ahead of the first store they spill, up to 40% longer.)
 struct Gamma8 {
@@ -89,13 +89,14 @@ __device__ __forceinline__ uint4 norm_rotate(uint4 x, const Gamma8& g, float r,
 // token-major inputs, so the warp walks them as 16-byte vectors; lane l always
 // holds vector l mod (d/8) of a head row, i.e. the same four pairs for every
 // head, so its cos/sin come from the tables once per token.
-// Two instances (the RMSNorm of K and Q has a kernel of its own).  kWave
-// holds the kernel to 64 registers (loads in batches of two), so four
+// kWave holds the kernel to 64 registers (loads in batches of two), so four
 // 256-thread blocks fit an SM and a launch of one 4680-token node (585
 // blocks) runs in a single wave: such a launch is bound by memory latency,
 // and occupancy is what hides it.  Larger launches loop over their tokens
 // and do better with batches of four at two blocks per SM.
-template <bool kWave>
+// kNorm: the RMSNorm of K (and Q) in front, for the launches that
+// launch_rope_kv gives to this kernel rather than to rope_norm_kernel.
+template <bool kNorm, bool kWave>
 __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __grid_constant__ RopeParams p) {
   const int lane = threadIdx.x & 31;
   const int vpr = p.d >> 3;                        // 16-byte vectors per (token, head) row
@@ -136,6 +137,25 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
     }
     const size_t in_tok = (size_t)tok * per_tok * 8;
     const size_t out_slot = ((size_t)nd.slot * 2 * p.H) * p.Tpad;  // row of (slot, K, head 0)
+    // RMSNorm scale of the token's K and Q vectors: a pass over the rows and a
+    // warp reduction; the pass below reads them again from L1 or L2.
+    float rk = 1.0f, rq = 1.0f;
+    if constexpr (kNorm) {
+      float sk = 0.0f, sq = 0.0f;
+      for (int v = lane; v < per_tok; v += 32) {
+        const size_t off = in_tok + (size_t)v * 8;
+        sk += sumsq8(*reinterpret_cast<const uint4*>(kin + off));
+        if (qio) sq += sumsq8(*reinterpret_cast<const uint4*>(qio + off));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sk += __shfl_xor_sync(0xffffffffu, sk, o);
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      }
+      const float inv_n = 1.0f / (float)(per_tok * 8);
+      rk = __frsqrt_rn(__fmaf_rn(sk, inv_n, p.norm_eps));
+      rq = __frsqrt_rn(__fmaf_rn(sq, inv_n, p.norm_eps));
+    }
     // Batches of kBatch vectors per lane: every load of a batch is issued
     // before any of its stores (q is rotated in place, so without the split
     // the compiler keeps each iteration's loads behind the previous stores).
@@ -144,6 +164,7 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
     constexpr int kBatch = kWave ? 2 : 4;
     for (int v0 = lane; v0 < per_tok; v0 += 32 * kBatch) {
       uint4 kv[kBatch], vv[kBatch], qv[kBatch];
+      Gamma8 next{};  // the gammas of the next vector to be stored
 #pragma unroll
       for (int j = 0; j < kBatch; ++j) {
         const int v = v0 + 32 * j;
@@ -154,23 +175,34 @@ __global__ void __launch_bounds__(256, kWave ? 4 : 2) rope_kv_kernel(const __gri
           qv[j] = qio ? *reinterpret_cast<const uint4*>(qio + in_off) : make_uint4(0, 0, 0, 0);
         }
       }
+      if constexpr (kNorm) next = gamma_at(p.gamma_k, v0);
+      auto turn = [&](uint4 x, const Gamma8& g, float r) {
+        if constexpr (kNorm) return norm_rotate(x, g, r, cs);
+        return make_uint4(rotate_pair(x.x, cs[0].x, cs[0].y), rotate_pair(x.y, cs[1].x, cs[1].y),
+                          rotate_pair(x.z, cs[2].x, cs[2].y), rotate_pair(x.w, cs[3].x, cs[3].y));
+      };
 #pragma unroll
       for (int j = 0; j < kBatch; ++j) {
         const int v = v0 + 32 * j;
         if (v >= per_tok) break;
         const int h = v >> vshift;
         const size_t in_off = in_tok + (size_t)v * 8;
-        uint32_t kw[4] = {kv[j].x, kv[j].y, kv[j].z, kv[j].w};
-        uint32_t qw[4] = {qv[j].x, qv[j].y, qv[j].z, qv[j].w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          kw[k] = rotate_pair(kw[k], cs[k].x, cs[k].y);
-          qw[k] = rotate_pair(qw[k], cs[k].x, cs[k].y);
-        }
         __nv_bfloat16* kdst = cache + ((out_slot + (size_t)h * p.Tpad + u) * p.d + c8 * 8);
-        *reinterpret_cast<uint4*>(kdst) = make_uint4(kw[0], kw[1], kw[2], kw[3]);
+        const bool more = j + 1 < kBatch && v + 32 < per_tok;
+        Gamma8 g = next;  // of this vector's K, then of its Q
+        if constexpr (kNorm) {
+          if (qio)
+            next = gamma_at(p.gamma_q, v);
+          else if (more)
+            next = gamma_at(p.gamma_k, v + 32);
+        }
+        *reinterpret_cast<uint4*>(kdst) = turn(kv[j], g, rk);
         *reinterpret_cast<uint4*>(kdst + kv_stride) = vv[j];
-        if (qio) *reinterpret_cast<uint4*>(qio + in_off) = make_uint4(qw[0], qw[1], qw[2], qw[3]);
+        if (qio) {
+          g = next;
+          if (kNorm && more) next = gamma_at(p.gamma_k, v + 32);
+          *reinterpret_cast<uint4*>(qio + in_off) = turn(qv[j], g, rq);
+        }
       }
     }
   }
@@ -310,24 +342,54 @@ cudaError_t launch_norm(const RopeParams& p, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s) {
-  const long long blocks = ((long long)p.n_nodes * p.T + 7) / 8;  // one warp per token
+  const long long tokens = (long long)p.n_nodes * p.T;
+  const long long sms = num_sms;
   const int per_tok = p.H * (p.d >> 3);  // 16-byte vectors, at most 2048
-  if (p.gamma_k != nullptr) {
-    // Few vectors a lane where that costs no bandwidth (a small launch is as
-    // long as one token takes: 320 tokens of 12 x 128, 5.4 us at six vectors,
-    // 4.0 at three), more where three would leave warps short of loads (40 x
-    // 128: 38 us at three, 35 at five; 16 x 64: 13.5 at three, 12.6 at four).
-    if (per_tok <= 64) return launch_norm<1, 2>(p, s);
-    if (per_tok <= 128) return launch_norm<1, 4>(p, s);
-    if (per_tok <= 192) return launch_norm<2, 3>(p, s);
-    if (per_tok <= 384) return launch_norm<4, 3>(p, s);
-    if (per_tok <= 640) return launch_norm<4, 5>(p, s);
-    if (per_tok <= 1280) return launch_norm<8, 5>(p, s);
-    return launch_norm<8, 8>(p, s);
-  }
   LaunchConfig l(dim3((unsigned)p.grid_blocks), 256, 0, s);
-  return blocks <= 4LL * num_sms ? cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<true>, p)
-                                 : cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<false>, p);
+  const bool wave = tokens <= 32 * sms;  // one warp a token, four blocks of eight warps per SM
+  if (p.gamma_k == nullptr)
+    return wave ? cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<false, true>, p)
+                : cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<false, false>, p);
+  const bool q = p.q != nullptr;
+  // The kernel that reads its rows twice with one warp a token is the faster
+  // one where the tokens fill most of a wave of it and rope_norm_kernel, with
+  // two to eight warps a token, needs the better part of two.
+  // At two blocks per SM (16 tokens): 2340 tokens of 16 x 128, K and V, 7.0 us
+  // against 8.6, with Q 9.0 against 11.5.  Below 8 or 12 tokens per SM the
+  // instances of two warps a token need one wave; past 448 vectors with Q, 768
+  // without, the second read no longer finds the rows in L1.
+  // At four (32 tokens): 4680 tokens of 13 x 128 with Q 15.3 us against 19.7,
+  // of 18 x 128 without 14.0 against 16.8.  At 24 tokens per SM the others fill
+  // their last wave (3120 tokens of 24 x 128, 14.4 against 13.0); narrower rows
+  // are no slower there on two warps a token, and with Q the rows that fill all
+  // lanes of <4, 3> are not either (24 x 128, three sets of buffers, 35.9
+  // against 34.3).
+  if (tokens > (q && per_tok > 192 && per_tok <= 256 ? 8 : 12) * sms && tokens <= 16 * sms &&
+      per_tok > 128 && per_tok <= (q ? 448 : 768))
+    return cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<true, false>, p);
+  if (tokens > 24 * sms && wave && per_tok > (q ? 192 : 256) && per_tok <= 448 &&
+      !(q && per_tok > 320 && per_tok <= 384))
+    return cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<true, true>, p);
+  // Few vectors a lane where that costs no bandwidth (a small launch is as
+  // long as one token takes: 320 tokens of 12 x 128, 5.4 us at six vectors,
+  // 4.0 at three), more where three would leave warps short of loads (40 x
+  // 128: 38 us at three, 35 at five; 16 x 64: 13.5 at three, 12.6 at four).
+  // From 129 to 768 vectors each step keeps two thirds of its lanes busy or
+  // more; in a wider one lanes idle through every load (18720 tokens of 13 x
+  // 128 with Q: 80 us on <4, 3>, 73 on <2, 4>; of 41 x 128 251 on <8, 5>, 206
+  // on <8, 3>).
+  if (per_tok <= 64) return launch_norm<1, 2>(p, s);
+  if (per_tok <= 128) return launch_norm<1, 4>(p, s);
+  if (per_tok <= 192) return launch_norm<2, 3>(p, s);
+  // within one wave of <4, 3>: 600 tokens of 16 x 128, 3.6 us, 4.0 on <2, 4>
+  if (per_tok <= 256 && tokens > 6 * sms) return launch_norm<2, 4>(p, s);
+  if (per_tok <= 384) return launch_norm<4, 3>(p, s);
+  if (per_tok <= 512) return launch_norm<4, 4>(p, s);
+  if (per_tok <= 640) return launch_norm<4, 5>(p, s);
+  // within two waves of <8, 5>: 600 tokens of 48 x 128 with Q, 9.0 us, 11.1 on <8, 3>
+  if (per_tok <= 768 && tokens > 4 * sms) return launch_norm<8, 3>(p, s);
+  if (per_tok <= 1280) return launch_norm<8, 5>(p, s);
+  return launch_norm<8, 8>(p, s);
 }
 
 }  // namespace sva

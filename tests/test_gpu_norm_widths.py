@@ -1,6 +1,8 @@
 """The RMSNorm + RoPE + cache write at the row widths where its kernel changes
 shape (one to eight warps a token, two to eight 16-byte vectors a lane), with
-token counts that leave part of the last block idle, with and without queries.
+token counts that leave part of the last block idle, with and without queries;
+and at the token counts, relative to the GPU's SMs, where it is given to the
+kernel that reads its rows twice, or just is not.
 
 Against fp64 torch: the result is rounded to bf16 once (2^-8 relative) after
 fp32 arithmetic, whose error is a few 2^-24 of the rotated pair's length (16
@@ -30,16 +32,31 @@ def _reference(x, gamma, t0, T, Wp, d, eps):
 
 
 @pytest.mark.parametrize("with_q", [False, True])
-@pytest.mark.parametrize("H,d", [(1, 64), (8, 64), (9, 64), (12, 128), (13, 128), (24, 128), (25, 128), (40, 128),
-                                 (41, 128), (128, 64), (80, 128), (81, 128), (128, 128)])
+@pytest.mark.parametrize("H,d", [(1, 64), (8, 64), (9, 64), (12, 128), (13, 128), (24, 128), (25, 128), (32, 128),
+                                 (33, 128), (40, 128), (41, 128), (48, 128), (128, 64), (80, 128), (81, 128),
+                                 (128, 128)])
 def test_norm_widths(H, d, with_q):
-    Hp, Wp, n, eps = 3, 15, 3, 1e-6
+    _check(H, d, with_q, 3, 15)
+
+
+# tokens per SM: just inside and just past the ranges in which the launch takes the other kernel
+@pytest.mark.parametrize("with_q", [False, True])
+@pytest.mark.parametrize("H,d", [(17, 64), (16, 128), (28, 128), (48, 128)])
+@pytest.mark.parametrize("per_sm,past", [(8, True), (12, True), (16, False), (16, True), (24, True), (32, False),
+                                         (32, True)])
+def test_norm_token_counts(per_sm, past, H, d, with_q):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    _check(H, d, with_q, 1, per_sm * sms // 3 + past, device="cuda")
+
+
+def _check(H, d, with_q, Hp, Wp, device="cpu"):
+    n, eps = 3, 1e-6
     T = Hp * Wp
     cache = sva.Cache(sva.make_geometry(H, d, 1, Hp, Wp, num_slots=n, pairs=rope_pairs_for(d), max_frames=16))
-    gen = torch.Generator().manual_seed(H * 1000 + d)
-    draw = lambda: (torch.randn((n, T, H, d), generator=gen) * 3).bfloat16().cuda()  # noqa: E731
+    gen = torch.Generator(device=device).manual_seed(H * 1000 + d)
+    draw = lambda: (torch.randn((n, T, H, d), generator=gen, device=device) * 3).bfloat16().cuda()  # noqa: E731
     k, v, q = draw(), draw(), draw()
-    gk, gq = (torch.rand(H * d, generator=gen).cuda() + 0.5 for _ in range(2))
+    gk, gq = (torch.rand(H * d, generator=gen, device=device).cuda() + 0.5 for _ in range(2))
     chunks = [2, 7, 11]
     slots = [cache.bind(0, c, 1) for c in chunks]
     nodes = [dict(seq=0, chunk=c, level=1, own_slot=s) for c, s in zip(chunks, slots)]
