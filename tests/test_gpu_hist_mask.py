@@ -15,7 +15,7 @@ from tests import _parity as P
 
 pytestmark = pytest.mark.gpu
 
-# T = 1024 in 4 frames, 2 history chunks, one head: 4 work units split 4 ways
+# T = 1024 in 4 frames, 2 history chunks, one head: 4 work units, each split over a cluster
 SPLITS = I.Workload(name="splitshist", seed=17, F=4, Hp=16, Wp=16, H=1, d=128, K=2, W=2,
                     policy="prog", nodes=((0, 3, 1),), prefilled=((0, 1, 0), (0, 2, 0)),
                     sparse=0.5, within="frame_causal",

@@ -11,9 +11,7 @@ from tests import _parity as P
 pytestmark = pytest.mark.gpu
 
 # One node, one head, T = 1024 in four frames of 256 tokens, one history
-# chunk: 4 work units of 16 key tiles, split 4 ways, so a key range starts
-# inside the own chunk past the frames of the first rows (which then see no
-# key in that range).
+# chunk: 4 work units of up to 16 key tiles, each split over a cluster of CTAs.
 SPLITFC = I.Workload(name="splitfc", seed=12, F=4, Hp=16, Wp=16, H=1, d=128, K=2, W=1,
                      policy="prog", nodes=((0, 2, 1),), prefilled=((0, 1, 0),),
                      within="frame_causal", description="split + frame-causal edge case")
@@ -32,11 +30,12 @@ def _all_rows(oracle_mod, w):
     step.close()
 
 
-# T = 1000 in 10 frames of 100 tokens, one history chunk: 4 work units of 16
-# key tiles split 4 ways.  The range of own tiles 4-7 (keys 512..1023) holds
-# no visible key for rows 400..499 but some for rows 500..511, which share a
-# warp with rows 496..499: rows whose max is still -inf in a warp where others
-# rescale (the softmax must not form -inf - -inf).
+# T = 1000 in 10 frames of 100 tokens, one history chunk: 4 work units of 11 to
+# 16 key tiles, each split over a cluster of four CTAs.  The second range of rows
+# 256..511 (13 key tiles) starts at own tile 3 (keys 384..511), of which rows up
+# to 299 see nothing and rows from 300 on see some keys; rows 288..303 share a
+# warp, so rows whose max is still -inf stand beside others that rescale (the
+# softmax must not form -inf - -inf).
 SPLITFC_WARP = I.Workload(name="splitfcwarp", seed=18, F=10, Hp=10, Wp=10, H=1, d=128, K=2, W=1,
                           policy="prog", nodes=((0, 2, 1),), prefilled=((0, 1, 0),),
                           within="frame_causal", description="masked and visible rows in one warp")

@@ -11,8 +11,8 @@ from tests import _parity as P
 pytestmark = pytest.mark.gpu
 
 # One node, one head, T = 1024 (8 tiles), two history chunks: 24 key tiles
-# over 4 work units, split 4 ways, so split ranges of a sparse mask can be
-# short or empty.
+# over 4 work units, each split over a cluster of CTAs, so that ranges of a sparse
+# mask can be short or empty.
 SPLITS = I.Workload(name="splits", seed=14, F=4, Hp=16, Wp=16, H=1, d=128, K=2, W=2,
                     policy="prog", nodes=((0, 3, 1),), prefilled=((0, 1, 0), (0, 2, 0)),
                     sparse=0.4, description="split + block-sparse edge cases")

@@ -1,6 +1,8 @@
-"""Key-range splits with the on-device merge: the split computation agrees
-with the oracle and with the unsplit computation, and the arrival counters
-are left at zero for the next launch."""
+"""Key-range splits with the on-device merge, inside a cluster (split4) and
+through the workspace (clean1): the split computation agrees with the oracle
+and with the unsplit computation, and the workspace's arrival counters are left
+at zero for the next launch.  Workspace merges of more ranges and with masks are
+in test_gpu_ws_merge.py."""
 import numpy as np
 import pytest
 import torch
@@ -11,7 +13,7 @@ from tests import _parity as P
 pytestmark = pytest.mark.gpu
 
 # 1 node, 2 heads, T = 240 (ragged query and key tiles), clean history of 7
-# chunks: 2 work units of 16 key tiles each, so the library splits them 4 ways.
+# chunks: 2 work units of 16 key tiles each, each split over a cluster of CTAs.
 SPLIT4 = I.Workload(name="split4", seed=9, F=1, Hp=8, Wp=30, H=2, d=128, K=4, W=7,
                     policy="clean", nodes=((0, 9, 4),),
                     prefilled=tuple((0, c, 0) for c in range(2, 9)),
@@ -30,7 +32,7 @@ def _run(w, inp, workspace):
     return step, q, out, lse
 
 
-def test_four_way_split_matches_oracle(oracle_mod):
+def test_cluster_split_matches_oracle(oracle_mod):
     w = SPLIT4
     inp = I.generate(w)
     step, q, out, lse = _run(w, inp, workspace=True)
@@ -40,7 +42,7 @@ def test_four_way_split_matches_oracle(oracle_mod):
     for h in range(w.H):
         P.assert_close(got[:, h, :], ref[h], f"split4 head {h}")
         np.testing.assert_allclose(lse[0, h].cpu().numpy(), ref_lse[h], atol=2e-3, rtol=0)
-    # counters were reset: a second launch on the same workspace agrees bitwise
+    # a second launch with the same workspace agrees bitwise, and the cluster merge leaves its counters alone
     nodes, _ = step.node_table()
     again = torch.empty_like(out)
     step.cache.attend_nodes(nodes, q, again, None, step.scale, check=False)
