@@ -333,7 +333,8 @@ sva_status sva_attend_nodes_masked(sva_cache* c, const sva_node* nodes, int32_t 
  * the device (the softmax of Eq. 4 recombined
  * from per-range maxima and sums), which fills the GPU when a launch has
  * too few work units; results agree with the unsplit computation to
- * rounding. */
+ * rounding.  A long launch of sva_attend_nodes_masked with token masks also
+ * keeps there, for its own duration, which key tiles they leave anything of. */
 size_t sva_attend_workspace_bytes(const sva_cache* c);
 
 /* Attaches a caller-owned device buffer of at least

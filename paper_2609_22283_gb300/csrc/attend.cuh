@@ -306,13 +306,14 @@ __device__ __forceinline__ void record_timeout(const AttnParams& p, volatile int
   atomicCAS(p.status, kStatusOk, kStatusTimeout);
 }
 
-// Instances: kSparse = a block-sparse tile mask is walked (all ones when the
-// caller gives none); kOwn = a token-level mask inside the own chunk is
-// applied (only with kSparse); kCluster = every unit is split over the CTAs of
-// one cluster, which merge through their shared memory.  Each extra feature
-// costs the per-tile loop, so a launch takes the leanest instance that covers
-// it.
-template <int D, bool kSparse, bool kOwn, bool kCluster>
+// Instances: kSparse = a bitmap of key tiles is walked: those of the caller's
+// tile mask (all without one) that the token masks leave anything of, where
+// the launch scanned them; kToken = token masks, of the own chunk or the
+// history or both, are applied (only with kSparse); kCluster = every unit is
+// split over the CTAs of one cluster, which merge through their shared memory.
+// Each extra feature costs the per-tile loop, so a launch takes the leanest
+// instance that covers it.
+template <int D, bool kSparse, bool kToken, bool kCluster>
 __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_constant__ AttnParams p) {
   using C = AttnCfg<D>;
   extern __shared__ uint8_t smem_raw[];
@@ -827,8 +828,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     for (int x = 0; x < NT; ++x) {
       const int u = (qt0 + (C::kOwnTile ? b_own : x)) * kTile + row;
       const size_t qrow = (size_t)nd.q_index * p.T + u;
-      own_row[x] = kOwn && p.own_mask && u < p.T ? p.own_mask + qrow * p.own_words + half * 2 : nullptr;
-      hist_row[x] = kOwn && p.hist_mask && u < p.T
+      own_row[x] =
+          kToken && p.own_mask && u < p.T ? p.own_mask + qrow * p.own_words + half * 2 : nullptr;
+      hist_row[x] = kToken && p.hist_mask && u < p.T
                         ? p.hist_mask + qrow * p.hist_states * p.hist_words + half * 2
                         : nullptr;
     }
@@ -889,7 +891,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         // tile needs no max tree.  Tiles that can hold masked keys (a slot's
         // ragged last tile, the own chunk under frame causality, token masks)
         // take mask_tile; the test is the same for every thread.
-        if (kOwn || valid_tile < kTile || own_fc) {
+        if (kToken || valid_tile < kTile || own_fc) {
           // own-chunk tile under frame causality: keys up to the end of this
           // row's latent frame are visible (tile 0, frame 0, always is)
           const int valid = own_fc ? min(valid_tile, frame_end[0] - t * kTile) : valid_tile;
@@ -898,11 +900,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           if (valid_tile < kTile || own_fc)
 #pragma unroll
             for (int c = 0; c < NC; ++c) w[c] &= first_bits(valid - c * 32);
-          if constexpr (!kOwn) mask_tile(s, w, m_part, m[0], sl2);
+          if constexpr (!kToken) mask_tile(s, w, m_part, m[0], sl2);
         }
         float m_new = fmaxf(m[0], m_part * sl2);
         bool move = __any_sync(0xffffffffu, m_new > m[0] + kRescaleThreshold) != 0;
-        if constexpr (kOwn) {
+        if constexpr (kToken) {
           if (move) {  // m_part was an upper bound: hidden keys counted
             m_new = fmaxf(m[0], max_visible(s, w) * sl2);
             move = __any_sync(0xffffffffu, m_new > m[0] + kRescaleThreshold) != 0;
@@ -947,7 +949,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
         for (int e = 0; e < 32; e += 2) {
           float x0, x1;
           ffma2(x0, x1, __uint_as_float(sc[e]), __uint_as_float(sc[e + 1]), sl2x2, negm);
-          if constexpr (kOwn) {
+          if constexpr (kToken) {
             if (!((wc >> e) & 1u)) x0 = -INFINITY;
             if (!((wc >> (e + 1)) & 1u)) x1 = -INFINITY;
           }
@@ -975,7 +977,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       uint32_t ow[NC];  // token masks: the bits of key tile kt
 #pragma unroll
       for (int c = 0; c < NC; ++c) ow[c] = ~0u;
-      if constexpr (kOwn)
+      if constexpr (kToken)
         if (my_tiles > 0) token_bits(0, kt, ow);
       for (int i = 0; ok && i < my_tiles; ++i) {
         const int kt_next = sparse ? walk.next() : next_kt(kt);
@@ -996,7 +998,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           uint32_t w[NC];  // token masks: the visible keys
           ok = row_max(i, s, cmax, ow, w);
           if (!ok) break;
-          if constexpr (kOwn)
+          if constexpr (kToken)
             if (i + 1 < my_tiles) token_bits(0, kt_next, ow);
           const uint64_t negm = neg_max();
           uint64_t acc[4] = {0, 0, 0, 0};
@@ -1010,7 +1012,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           tc_fence_before();
           add_sum(acc);
           o_has[0] = true;
-        } else if constexpr (kOwn) {
+        } else if constexpr (kToken) {
           if (i + 1 < my_tiles) token_bits(0, kt_next, ow);
         }
         mbar_arrive(p_bar);
@@ -1029,7 +1031,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       for (int b = 0; b < 2; ++b) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) ow[b][c] = ~0u;
-        if constexpr (kOwn)
+        if constexpr (kToken)
           if (n_tiles > 0) token_bits(b, kt, ow[b]);
       }
       for (int i = 0; ok && i < n_tiles; ++i, kt = kt_next) {
@@ -1056,7 +1058,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           if (sparse && !((attends >> b) & 1u)) {
             // query tile b skips this key tile: no S was computed, no P is due
             mbar_arrive(&bars.p_full[b]);
-            if constexpr (kOwn)
+            if constexpr (kToken)
               if (i + 1 < n_tiles) token_bits(b, kt_next, ow[b]);
             continue;
           }
@@ -1080,7 +1082,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           // that changes them and one that does not had their registers copied
           // where the two meet (451 us against 400 with random masks).
           uint32_t wm[2] = {~0u, ~0u};
-          if (kOwn || valid_tile < kTile || own_fc) {
+          if (kToken || valid_tile < kTile || own_fc) {
             // own-chunk tile under frame causality: keys up to the end of this
             // row's latent frame are visible (tile 0, frame 0, always is)
             const int valid = own_fc ? min(valid_tile, frame_end[b] - t * kTile) : valid_tile;
@@ -1090,7 +1092,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
               w[0] &= first_bits(vrel);
               w[1] &= first_bits(vrel - 32);
             }
-            if constexpr (kOwn) {
+            if constexpr (kToken) {
               wm[0] = w[0];
               wm[1] = w[1];
               if (i + 1 < n_tiles) token_bits(b, kt_next, ow[b]);
@@ -1101,7 +1103,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           float m_tile = fmaxf(m_part, __shfl_xor_sync(0xffffffffu, m_part, 16)) * sl2;
           float m_new = fmaxf(m[b], m_tile);
           bool move = __any_sync(0xffffffffu, m_new > m[b] + kRescaleThreshold) != 0;
-          if constexpr (kOwn) {
+          if constexpr (kToken) {
             // m_part is the maximum with the hidden keys, an upper bound: only
             // where that could move m is the one over the visible keys taken
             if (move) {
@@ -1149,7 +1151,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
             for (int e = 0; e < 32; e += 2) {
               float x0, x1;
               ffma2(x0, x1, __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]), sl2x2, negm);
-              if constexpr (kOwn) {
+              if constexpr (kToken) {
                 if (!((wm[c] >> e) & 1u)) x0 = -INFINITY;
                 if (!((wm[c] >> (e + 1)) & 1u)) x1 = -INFINITY;
               }
@@ -1471,9 +1473,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
 }  // namespace
 
 // The kernel's instances are compiled in three units (attend_dense.cu,
-// attend_cluster.cu, attend_masked.cu): in one, the machine code of the dense
-// instance lay differently whenever another instance changed, and its speed
-// with it (a 4680-token layer between 367 and 381 us for the same source).
+// attend_cluster.cu, attend_masked.cu), because in one the speed of the dense
+// instance was seen to change with the code of the others (a 4680-token layer
+// between 367 and 381 us for the same source of its own).  Why is not known:
+// after a change to this file, time the dense launches too, whichever instance
+// it was for.
 using AttendKernel = void (*)(const AttnParams);
 
 // Without splits inside clusters: dense; block-sparse, and with token masks.

@@ -11,10 +11,12 @@
 // Bound by the read of the masks: one block per (node, query tile, key state),
 // two rows per warp at a time, 32 words (8 key tiles) a load, up to sixteen
 // loads in flight.  A warp whose rows so far have set a bit in every tile
-// stops reading, so dense random masks cost a few rows per block.  One 4680-token node, 3 history
-// states, bits within 6 patch rows and columns (11 MB of masks): 7 us before
-// an attention launch that takes 394 us over every key tile and 262 us over the
-// 58% of them that keep a bit for the query-tile pair.
+// stops reading, so dense random masks cost a few rows per block.  Times (one
+// launch under ncu): one 4680-token node, 3 history states, bits within 6 patch
+// rows and columns (11 MB of masks) 7 us, random bits of the same size 4 us;
+// 8220 tokens, one history state, bits within 12 rows and columns (17 MB) 9 us.
+// The first two are followed by an attention launch of 259 us over the 58% of
+// key tiles that keep a bit for their query-tile pair, and of 388 us over all.
 #include <cuda_runtime.h>
 
 #include "internal.h"

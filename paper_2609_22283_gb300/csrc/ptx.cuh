@@ -23,19 +23,6 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   return t;
 }
 
-__device__ __forceinline__ uint32_t elect_one_sync() {
-  uint32_t pred = 0;
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " .reg .b32 r;\n"
-      " elect.sync r|p, 0xffffffff;\n"
-      " selp.u32 %0, 1, 0, p;\n"
-      "}\n"
-      : "=r"(pred));
-  return pred;
-}
-
 // ---------------------------------------------------------------- launches
 //
 // Programmatic dependent launch: a kernel launched with the attribute may start
@@ -153,15 +140,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar,
-                                            int32_t c0, int32_t c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(c0), "r"(c1)
-      : "memory");
 }
 
 __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* map, uint64_t* bar,
@@ -325,47 +303,14 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo_byt
   return d;
 }
 
+// Warp-wide calls: every lane of a converged warp executes them and elect.sync
+// picks the issuing lane (the lowest active one, so always the same thread: a
+// commit tracks the MMAs of the thread that issues it).  A loop that stays
+// warp-uniform keeps descriptors and TMEM addresses in the uniform datapath;
+// issuing from a lane-0-only branch was measured about 8% slower end to end in
+// the attention kernel.
+
 // D[tmem] (+)= A[smem] * B[smem]
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                       uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-      "}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// D[tmem] (+)= A[tmem] * B[smem]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
-                                       uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n"
-      " .reg .pred p;\n"
-      " setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
-      "}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Arrives once on `bar` when every tcgen05 operation issued so far by this
-// thread has completed.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
-      : "memory");
-}
-
-// Warp-wide forms of the three calls above: every lane of a converged warp
-// executes them and elect.sync picks the issuing lane (the lowest active one,
-// so always the same thread: a commit tracks the MMAs of the thread that
-// issues it).  A loop that stays warp-uniform keeps descriptors and TMEM
-// addresses in the uniform datapath; issuing from a lane-0-only branch was
-// measured about 8% slower end to end in the attention kernel.
 __device__ __forceinline__ void mma_ss_warp(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -379,6 +324,7 @@ __device__ __forceinline__ void mma_ss_warp(uint32_t d_tmem, uint64_t a_desc, ui
       : "memory");
 }
 
+// D[tmem] (+)= A[tmem] * B[smem]
 __device__ __forceinline__ void mma_ts_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
                                             uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -443,6 +389,8 @@ __device__ __forceinline__ void mma_ts_warp_x8(uint32_t d_tmem, uint32_t a_tmem,
       : "memory");
 }
 
+// Arrives once on `bar` when every tcgen05 operation that the issuing lane
+// issued so far has completed.
 __device__ __forceinline__ void mma_commit_warp(uint64_t* bar) {
   asm volatile(
       "{\n"
@@ -472,9 +420,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr));
 }
 
-// Waits for this thread's outstanding tensor-memory loads.  Taking the
-// registers as read-write operands keeps the compiler from hoisting their
-// uses above the wait.
 // tmem_ld32 that also returns the maximum of the 32 loaded fp32 values
 // (tcgen05.ld.red, sm_103a): a row max of S without a max tree in registers.
 // `mx`, like the registers, is valid only after a tcgen05.wait::ld that
@@ -488,6 +433,9 @@ __device__ __forceinline__ void tmem_ld32_max(uint32_t taddr, uint32_t (&r)[32],
       : "r"(taddr));
 }
 
+// Waits for this thread's outstanding tensor-memory loads.  Taking the
+// registers as read-write operands keeps the compiler from hoisting their
+// uses above the wait.
 __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : SVA_RW8(0), SVA_RW8(8), SVA_RW8(16), SVA_RW8(24)

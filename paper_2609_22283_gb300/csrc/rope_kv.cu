@@ -376,7 +376,7 @@ cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s) {
   // 128: 38 us at three, 35 at five; 16 x 64: 13.5 at three, 12.6 at four).
   // From 129 to 768 vectors each step keeps two thirds of its lanes busy or
   // more; in a wider one lanes idle through every load (18720 tokens of 13 x
-  // 128 with Q: 80 us on <4, 3>, 73 on <2, 4>; of 41 x 128 251 on <8, 5>, 206
+  // 128 with Q: 80 us on <4, 3>, 69 on <2, 4>; of 41 x 128 251 on <8, 5>, 206
   // on <8, 3>).
   if (per_tok <= 64) return launch_norm<1, 2>(p, s);
   if (per_tok <= 128) return launch_norm<1, 4>(p, s);

@@ -268,9 +268,15 @@ size_t ws_total_bytes(const sva_cache* c) {
 }
 
 // Workspace items that the scan of token masks may take from the split
-// partials.  A plan splits at most one wave of units 4 ways, so it leaves 4 of
-// the 4 waves of items over.
+// partials.  A split of s ranges is made only where they need fewer than s
+// waves, so a plan takes at most 3 * num_sms of the 4 * num_sms items and these
+// do not change it.
 constexpr long long kScanItems = 4;
+// Walks of a key tile by a query-tile pair from which token masks are scanned:
+// about 100 us of attention on 152 SMs (1.2 us a walk), whatever the masks then
+// leave of them.  The scan takes 4 to 9 us (mask_scan.cu), by the masks' bytes
+// and not by the heads: a launch at the line pays 4 to 9% where they empty no
+// tile.
 constexpr long long kScanMinTiles = 12000;
 
 // Fewest key tiles a work unit of node i walks: all of its slots' tiles,
@@ -817,8 +823,7 @@ sva_status attend(sva_cache* c, const sva_node* nodes, int32_t n_nodes, const vo
   long long cap = (scratch == Scratch::kStatic || c->ws != nullptr) ? ws_items(c) : 0;
   // A launch with token masks scans them first for the key tiles they leave
   // anything of, when a workspace can take the result and the launch is long
-  // enough for the scan's 3-5 us to be lost in it: kScanMinTiles walks of a
-  // key tile by a query-tile pair, about 100 us of attention.
+  // enough (kScanMinTiles).
   int max_states = 1;
   for (int i = 0; i < n_nodes; ++i) max_states = std::max(max_states, 1 + nodes[i].n_ctx);
   size_t scan_bytes = 0;
