@@ -123,3 +123,16 @@ def test_two_way_merge_frame_causal():
     frame = torch.arange(a.T, device="cuda") // a.fr
     a.check(out, lse, (frame[None, :] <= frame[:, None]).expand(2, -1, -1), [0, 25, 26, 28])
     a.c.close()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_equal_cost_goes_to_clusters(d):
+    """48 units of 24 key tiles: three ranges through the workspace and clusters of two cost the plan the
+    same, and clusters leave the workspace alone."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms != 152:
+        pytest.skip("the units are chosen for 152 SMs")
+    a = Launch(1, 16, 16, 24, d, 2, 11, grow=5.0)
+    out, lse = a.run(0)
+    a.check(out, lse, torch.ones((2, a.T, 12 * a.T), dtype=torch.bool, device="cuda"), [0, 11, 23])
+    a.c.close()
