@@ -323,6 +323,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
   __shared__ uint32_t tmem_base_sh;
   __shared__ volatile int abort_flag;
   __shared__ int last_split;
+  __shared__ float range_lost;  // kCluster: not 0 once a key range of the unit has timed out
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -397,6 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
     prefetch_tmap(&p.tmap_q);
     prefetch_tmap(&p.tmap_kv);
     abort_flag = 0;
+    if constexpr (kCluster) range_lost = 0.0f;
     mbar_init(&bars.q_full, 1);
     mbar_init(&bars.o_final, 2);  // one commit per MMA issuer
     mbar_init(&bars.drain, 2);
@@ -1193,8 +1195,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
       // over the unit's CTAs (131 KB out and in per CTA at D = 128, whatever
       // ns), needs no workspace, and costs two cluster barriers instead of
       // stores to L2, a fence, an atomic and the last CTA's reads.  A range
-      // that timed out sends l = -1 in place of its rows, and no owner writes
-      // those: what its partial would have been is not in shared memory.
+      // that timed out sets every CTA's range_lost in place of its rows, and
+      // no owner stores the unit: what the range's partial would have been is
+      // not in shared memory.
       constexpr int kGroups8 = D / 8;
       const int per = (kGroups8 + ns - 1) / ns;  // column groups per owner
       const uint32_t data = smem_u32(smem);
@@ -1239,43 +1242,32 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
               st_cluster_f32(dst + 1024, l_row[x]);
             }
         }
-      } else {
-#pragma unroll
-        for (int x = 0; x < NT; ++x)
-          if (half == 0)
-            for (int k = 0; k < ns; ++k) {
-              const int r = (C::kOwnTile ? b_own : x) * 128 + row;
-              const uint32_t dst = mapa_shared(ml + (uint32_t)(split * 2048 + r * 4), (uint32_t)k);
-              st_cluster_f32(dst, -INFINITY);
-              st_cluster_f32(dst + 1024, -1.0f);
-            }
+      } else if (lane < ns) {
+        st_cluster_f32(mapa_shared(smem_u32(&range_lost), (uint32_t)lane), 1.0f);
       }
       __syncwarp();
       cluster_sync();  // every partial has arrived; nothing is read from another CTA after this
       const int r = threadIdx.x - 128;  // this thread's row of the pair
       const int token = qt0 * kTile + r;
-      if (ok && token < p.T && r < nb * kTile) {
+      if (ok && ld_shared_f32(smem_u32(&range_lost)) == 0.0f && token < p.T && r < nb * kTile) {
         float M = -INFINITY;
         for (int k = 0; k < ns; ++k) M = fmaxf(M, ld_shared_f32(ml + (uint32_t)(k * 2048 + r * 4)));
         const float M_sub = (M == -INFINITY) ? 0.0f : M;  // every range empty: O = 0
         float w[kMaxClusterSplit];
         float L = 0.0f;
-        bool whole = true;  // every range has sent this row
 #pragma unroll
         for (int k = 0; k < kMaxClusterSplit; ++k) {
           w[k] = 0.0f;
           if (k < ns) {
             const uint32_t at = ml + (uint32_t)(k * 2048 + r * 4);
-            const float l_k = ld_shared_f32(at + 1024);
-            whole = whole && !(l_k < 0.0f);
-            w[k] = l_k * ex2(ld_shared_f32(at) - M_sub);
+            w[k] = ld_shared_f32(at + 1024) * ex2(ld_shared_f32(at) - M_sub);
             L += w[k];
           }
         }
         const float inv_L = L > 0.0f ? 1.0f / L : 0.0f;
         uint4* orow4 = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(p.out) +
                                                 (((size_t)nd.q_index * p.T + token) * p.H + h) * D);
-        for (int g = 0; whole && g < per && split * per + g < kGroups8; ++g) {
+        for (int g = 0; g < per && split * per + g < kGroups8; ++g) {
           float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int k = 0; k < kMaxClusterSplit; ++k) {
@@ -1292,7 +1284,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_kernel(const __grid_consta
           orow4[split * per + g] = make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]),
                                               pack_bf16(a[4], a[5]), pack_bf16(a[6], a[7]));
         }
-        if (whole && p.lse != nullptr && split == 0)
+        if (p.lse != nullptr && split == 0)
           p.lse[((size_t)nd.q_index * p.H + h) * p.T + token] = (M + __log2f(L)) * 0.69314718055994531f;
       }
     } else if (ns == 1) {
