@@ -359,15 +359,15 @@ cudaError_t launch_rope_kv(const RopeParams& p, int num_sms, cudaStream_t s) {
   // one where the tokens fill most of a wave of it and rope_norm_kernel, with
   // two to eight warps a token, needs the better part of two.
   // At two blocks per SM (16 tokens): 2340 tokens of 16 x 128, K and V, 7.0 us
-  // against 8.6, with Q 9.0 against 11.5.  Below 8 or 12 tokens per SM the
-  // instances of two warps a token need one wave; past 448 vectors with Q, 768
-  // without, the second read no longer finds the rows in L1.
-  // At four (32 tokens): 4680 tokens of 13 x 128 with Q 15.3 us against 19.7,
-  // of 18 x 128 without 14.0 against 16.8.  At 24 tokens per SM the others fill
-  // their last wave (3120 tokens of 24 x 128, 14.4 against 13.0); narrower rows
-  // are no slower there on two warps a token, and with Q the rows that fill all
-  // lanes of <4, 3> are not either (24 x 128, three sets of buffers, 35.9
-  // against 34.3).
+  // against 8.6, of 12 x 128 with Q 7.8 against 9.0.  Below 8 or 12 tokens per
+  // SM the instances of two warps a token need one wave; past 448 vectors with
+  // Q, 768 without, the second read no longer finds the rows in L1.
+  // At four (32 tokens): 4680 tokens of 18 x 128, K and V, 13.7 us against 16.6,
+  // with Q 20.8 against 24.6.  At 24 tokens per SM the others fill their last
+  // wave (3120 tokens of 24 x 128, 14.4 against 12.9); narrower rows are no
+  // slower there on two warps a token, and with Q the rows that fill all lanes
+  // of <4, 3> are not either (24 x 128, three sets of buffers, 35.9 against
+  // 34.2).
   if (tokens > (q && per_tok > 192 && per_tok <= 256 ? 8 : 12) * sms && tokens <= 16 * sms &&
       per_tok > 128 && per_tok <= (q ? 448 : 768))
     return cudaLaunchKernelEx(&l.cfg, rope_kv_kernel<true, false>, p);
